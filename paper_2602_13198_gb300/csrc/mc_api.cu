@@ -163,6 +163,12 @@ DevModel make_model(const mc_ctx *c) {
   m.kapA = c->kapA;
   m.kapI = c->kapI;
   m.kapH = c->kapH;
+  m.a2 = p.a * p.a;
+  m.twoa = 2.0 * p.a;
+  m.M2 = 2.0 * p.mass;
+  m.pi2hh = kPI * (1.0 - p.hslope);
+  m.hh_pi2 = (1.0 - p.hslope) / kPI;
+  m.d2th2 = -4.0 * kPI * kPI * (1.0 - p.hslope);
   m.dmass = df_const(m.mass);
   m.da = df_const(m.a);
   m.dx1_0 = df_const(m.x1_0);

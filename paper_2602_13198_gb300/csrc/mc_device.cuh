@@ -199,6 +199,27 @@ __device__ __forceinline__ int floor_frac(double f, double &frac) {
 // cell index and the fraction within it, FP64 coordinates
 __device__ __forceinline__ int zone_split(double f, double &frac) { return floor_frac(f, frac); }
 
+// 1 / x and 1 / sqrt(x) for positive normal x whose result is normal too: the hardware's 20-bit approximation
+// and one third-order step (Householder's for x^-1, x^-1/2: y <- y (1 + e + e^2) with e = 1 - x y, and
+// y <- y (1 + e/2 + 3 e^2/8) with e = 1 - x y^2), which leaves an error of order e^3 ~ 2^-60 before rounding.
+// Three and five FP64-pipe operations where the compiler's take about 5.5 and 6.4 (measured: 354 and 408
+// cycles a warp at 64 cycles per FP64 instruction on one SM partition).
+__device__ __forceinline__ double rcp_n(double x) {
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double e = fma(-x, y, 1.0);
+  return fma(y, fma(e, e, e), y);
+}
+__device__ __forceinline__ double rsqrt_n(double x) {
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double e = fma(-(x * y), y, 1.0);
+  return fma(fma(e, 0.375, 0.5) * e, y, y);
+}
+
+// x2 > 1/2
+__device__ __forceinline__ bool upper_half(double x) { return __double_as_longlong(x) > 0x3FE0000000000000LL; }
+
 // ---------------------------------------------------------------- model view passed to kernels
 struct DevModel {
   // metric and units
@@ -238,6 +259,7 @@ struct DevModel {
   int brems;              // thermal bremsstrahlung on
   df dmass, da, dx1_0, dx1_hi, dr_record, dr_capture;   // double-float splits for the mixed geodesic
   df dpi2hh, dhh_pi, dd2th;   // pi (1 - h), (1 - h) / (2 pi), -2 pi^2 (1 - h): the theta map in double-float
+  double a2, twoa, M2, pi2hh, hh_pi2, d2th2;   // a^2, 2 a, 2 M and the theta map's pi (1-h), (1-h) / pi, -4 pi^2 (1-h)
   const df *dtab;             // double-float function table (kDfTabN entries)
   float fidx1, fidx2, fidx3, fx2_0, fx3_0;   // FP32 grid constants for the double-float zone lookup
   // FP32 copies of model constants and tables read by the FP32 arithmetic (no FP64 conversions there)
@@ -623,16 +645,182 @@ __device__ __forceinline__ void accel(const GeoT<S> &G, const S k[4], S A[4]) {
   A[3] = -sdot(G.G13, w1, G.G33, w3);
 }
 
+// Kerr-Schild geometry at a point.  The metric is g = g0 + f l l with f = 2 M r / Sigma, the null covector
+// l = (1, 1, 0, -a sin^2) in (t, r, theta, phi) and a background g0 that is flat space in spheroidal
+// coordinates: ds0^2 = -dt^2 + dr^2 + Sigma dtheta^2 + (r^2 + a^2) sin^2 dphi^2 - 2 a sin^2 dr dphi, and
+// g^-1 = g0^-1 - f l l with l^a = (-1, 1, 0, 0).  The geodesic needs f, l and the shared factors below and
+// no metric component or derivative.  double is the scalar of the geodesic arithmetic: double, or df in the
+// mixed form (specialised below).
+struct Point {
+  double r, s, c;            // radius, sin and cos of theta
+  double dth, d2th;          // d theta / d x2, d^2 theta / d x2^2
+  double s2, sc, r2;         // sin^2, sin cos, r^2
+  double ir, idth;           // 1 / r, 1 / dth
+  double f;                  // 2 M r / Sigma
+  double sig, isig, is2;     // Sigma = r^2 + a^2 cos^2, its reciprocal, 1 / sin^2
+  double r2a2, as2;          // r^2 + a^2, a sin^2 (a != 0 only)
+  double q1h;                // (d ln f / d ln r) / 2 = 1/2 - r^2 / Sigma
+  double tr, asc2, scr2;     // 2 r, 2 a sin cos (a != 0 only), 2 sin cos (r^2 + a^2)
+};
+
+// Point geometry at (x1, x2).  theta is counted from the nearer pole (y = x2 or 1 - x2, exact for x2 in
+// [1/2, 1]), so that sin(theta) keeps its relative accuracy at both: theta/pi = y + (1-h)/(2 pi) sin(2 pi y),
+// and one more sincospi gives sin and cos of theta.  Reciprocals are taken one by one (three to four
+// operations each, see srcp), which costs less than one division and the products that split it.
+// KERR = false: the a = 0 (Schwarzschild) form, with the terms that vanish at a = 0 left out.
+template <bool KERR = true>
+__device__ __forceinline__ void point_eval(const DevModel &m, double x1, double x2, Point &G) {
+  const bool far = upper_half(x2);
+  const double y = far ? ssub(1.0, x2) : x2;
+  G.r = exp_t(m.ftab, x1);
+  double sp, cp;
+  sincospi_t(m.ftab, y, sp, cp);
+  if (m.hslope1) {
+    G.s = sp;
+    G.c = cp;
+    G.dth = kPI;
+    G.d2th = 0.0;
+    G.idth = 1.0 / kPI;
+  } else {
+    const double sc1 = smul(sp, cp);                                         // sin(2 pi y) / 2
+    G.dth = mad(m.pi2hh, smul(ssub(cp, sp), sadd(cp, sp)), kPI);   // pi (1 + (1-h) cos(2 pi y))
+    G.d2th = smul(m.d2th2, sc1);                     // -2 pi^2 (1-h) sin(2 pi y)
+    sincospi_t(m.ftab, mad(m.hh_pi2, sc1, y), G.s, G.c);
+    G.idth = rcp_n(G.dth);
+  }
+  if (far) {
+    G.c = -G.c;
+    G.d2th = -G.d2th;
+  }
+  G.s2 = smul(G.s, G.s);
+  G.sc = smul(G.s, G.c);
+  G.r2 = smul(G.r, G.r);
+  G.ir = rcp_n(G.r);
+  const double M2 = m.M2;
+  G.is2 = rcp_n(G.s2);
+  G.tr = stwice(G.r);
+  const double sc2 = stwice(G.sc);
+  if constexpr (KERR) {
+    const double a = m.a, a2 = m.a2;
+    const double a2c2 = smul(a2, smul(G.c, G.c));
+    G.sig = sadd(G.r2, a2c2);
+    G.isig = rcp_n(G.sig);
+    G.r2a2 = sadd(G.r2, a2);
+    G.as2 = smul(a, G.s2);
+    G.asc2 = smul(a, sc2);
+    G.q1h = smul(shalf(ssub(a2c2, G.r2)), G.isig);
+  } else {
+    G.sig = G.r2a2 = G.r2;
+    G.isig = rcp_n(G.r2);
+    G.q1h = -smul(shalf(G.r2), G.isig);
+  }
+  G.f = smul(smul(M2, G.r), G.isig);
+  G.scr2 = smul(sc2, G.r2a2);
+}
+
+// Metric and inverse metric components from the point geometry.
+template <bool KERR = true>
+__device__ __forceinline__ void metric_of(const DevModel &m, const Point &P, Geo &G) {
+  const double zero = 0.0;
+  const double opf = sadd(P.f, 1.0);
+  G.r = P.r;
+  G.sth = P.s;
+  G.cth = P.c;
+  G.g00 = ssub(P.f, 1.0);
+  G.g01 = smul(P.f, P.r);
+  G.g11 = smul(opf, P.r2);
+  G.g22 = smul(P.sig, smul(P.dth, P.dth));
+  G.G00 = -opf;
+  G.G01 = smul(P.f, P.ir);
+  G.G22 = smul(P.isig, smul(P.idth, P.idth));
+  G.G33 = smul(P.isig, P.is2);
+  const double rm = ssub(P.r, m.M2);
+  if constexpr (KERR) {
+    const double a = m.a;
+    G.g03 = -smul(P.as2, P.f);
+    G.g13 = -smul(smul(P.as2, opf), P.r);
+    G.g33 = smul(P.s2, mad(smul(a, P.as2), opf, P.sig));   // sin^2 (Sigma + a^2 sin^2 (1 + f))
+    G.G11 = smul(smul(mad(P.r, rm, m.a2), P.isig), smul(P.ir, P.ir));
+    G.G13 = smul(smul(a, P.isig), P.ir);
+  } else {
+    G.g03 = G.g13 = G.G13 = zero;
+    G.g33 = smul(P.s2, P.sig);
+    G.G11 = smul(smul(smul(P.r, rm), P.isig), smul(P.ir, P.ir));
+  }
+}
+
+// dk^mu/dlambda of a null geodesic in the internal coordinates (x1 = ln r, theta(x2)), from the
+// Euler-Lagrange equations d(g k)_mu = (1/2) d_mu g_ab k^a k^b, so dk = g^-1 F with F_mu = (1/2) d_mu g_ab k^a k^b
+// - (dg/dlambda k)_mu.  With g = g0 + f l l everything is written in f, l and the projection
+// L = l_a k^a = k^t + k^r - a sin^2 k^phi, with w = d(a sin^2)/dlambda, u = d(f L)/dlambda at fixed k and
+// Sd = dSigma/dlambda:
+//   F_t = -u, F_r = S - u, S = r (k_th^2 + sin^2 k_ph^2) + (1/2) f_r L^2 + w k_ph (= l^a F_a),
+//   F_ph = w (k^r + f L) + a sin^2 u - 2 k_ph (sin^2 r k^r + sin cos (r^2 + a^2) k_th),
+//   F_th = sin cos ((r^2 + a^2) k_ph^2 - a^2 k_th^2 + a^2 f L^2 / Sigma - 2 a k_ph (k^r + f L)) - Sd k_th,
+// then dk^t = u + f S, dk^r = ((r^2 + a^2) F_r + a F_ph) / Sigma - f S, dk^th = F_th / Sigma,
+// dk^ph = (a F_r + F_ph / sin^2) / Sigma, and dk^1 = dk^r / r - k^1 k^1, dk^2 = (dk^th - theta'' k^2 k^2) / theta'.
+// About 55 multiply-adds; contracting the metric's derivatives (14 of them, with 13 components) took
+// about 200 operations and kept all of them live across the predictor loop.  The FP64 pipe bounds these kernels
+// (one warp instruction per 64 cycles on each SM partition), so the count is the time: one shard of the 3-D
+// snapshot went from 539 to 442 ms in FP64 and from 401 to 303 ms in the split form with the network.  KERR = false leaves out the
+// terms that are exactly zero at a = 0 and nothing else, so that the two forms agree bit for bit there (a
+// batch runs every model in the general form).
+template <bool KERR = true>
+__device__ __forceinline__ void accel(const DevModel &m, const Point &G, const double k[4], double A[4]) {
+  const double k1 = k[1], kp = k[3];
+  const double kr = smul(G.r, k1), kh = smul(G.dth, k[2]);
+  const double kpp = smul(kp, kp), khh = smul(kh, kh);
+  const double th = mad(G.s2, kpp, khh);
+  const double r2k2 = smul(G.tr, kr);
+  double L = sadd(k[0], kr), Sd2 = r2k2, w, wp;
+  if constexpr (KERR) {
+    w = smul(G.asc2, kh);
+    wp = smul(w, kp);
+    L = nmad(G.as2, kp, L);
+    Sd2 = nmad(m.a, w, r2k2);            // dSigma/dlambda
+  }
+  const double fL = smul(G.f, L), fLL = smul(fL, L);
+  const double gg = nmad(G.isig, Sd2, k1);                   // (df/dlambda) / f
+  double u, S0, Fp, br;
+  if constexpr (KERR) {
+    u = smul(G.f, msub(gg, L, wp));
+    S0 = mad(G.ir, smul(G.q1h, fLL), mad(G.r, th, wp));
+  } else {
+    u = smul(G.f, smul(gg, L));
+    S0 = mad(G.ir, smul(G.q1h, fLL), smul(G.r, th));
+  }
+  const double Fr = ssub(S0, u), fS = smul(G.f, S0);
+  const double Fc = dot2(G.s2, r2k2, G.scr2, kh);
+  if constexpr (KERR) {
+    const double v = sadd(kr, fL);
+    Fp = nmad(kp, Fc, dot2(w, v, G.as2, u));
+    br = nmad(smul(m.twoa, kp), v, dot2(m.a2, msub(G.isig, fLL, khh), G.r2a2, kpp));
+  } else {
+    Fp = -smul(kp, Fc);
+    br = smul(G.r2a2, kpp);
+  }
+  const double Fh = nmad(Sd2, kh, smul(G.sc, br));
+  A[0] = sadd(u, fS);
+  A[2] = smul(nmad(smul(G.d2th, k[2]), k[2], smul(G.isig, Fh)), G.idth);
+  if constexpr (KERR) {
+    const double a = m.a;
+    A[1] = nmad(k1, k1, smul(msub(G.isig, dot2(G.r2a2, Fr, a, Fp), fS), G.ir));
+    A[3] = smul(G.isig, dot2(Fp, G.is2, a, Fr));
+  } else {
+    A[1] = nmad(k1, k1, smul(msub(G.isig, smul(G.r2a2, Fr), fS), G.ir));
+    A[3] = smul(G.isig, smul(Fp, G.is2));
+  }
+}
+
 // Step size (reading; the paper gives none): each internal coordinate moves at most eps_geo of
 // its scale (1 for ln r and phi, the distance to the nearer pole for x2).
 template <typename S = double>
 __device__ __forceinline__ S stepsize(const DevModel &m, const S X[4], const S K[4]) {
-  // 1 / (1/d1 + 1/d2 + 1/d3) with d1 = eps/(|k1|+S), d2 = eps x2n/(|k2|+S), d3 = eps/(|k3|+S)
-  // = eps x2n / ((|k1| + |k3|) x2n + |k2|): one division
-  const double SMALL = 1e-40;
-  double x2n = dmin_nn(fabs(X[2]), fabs(1.0 - X[2]));
-  double den = ((fabs(K[1]) + SMALL) + (fabs(K[3]) + SMALL)) * x2n + (fabs(K[2]) + SMALL);
-  return m.eps_geo * x2n / den;
+  // 1 / (1/d1 + 1/d2 + 1/d3) with d1 = eps/|k1|, d2 = eps x2n/|k2|, d3 = eps/|k3|
+  // = eps x2n / ((|k1| + |k3|) x2n + |k2|): one reciprocal
+  const double x2n = dmin_nn(fabs(X[2]), fabs(__dsub_rn(1.0, X[2])));
+  const double den = fma(__dadd_rn(fabs(K[1]), fabs(K[3])), x2n, __dadd_rn(fabs(K[2]), 1e-40));
+  return __dmul_rn(__dmul_rn(m.eps_geo, x2n), rcp_n(den));
 }
 
 // Double-float step size: the same rule in double-float, so that the steps land where the FP64
@@ -915,7 +1103,7 @@ __device__ __forceinline__ bool outside_radially(const DevModel &m, const df X[4
 template <typename T, typename S, bool F32IDX = false>
 __device__ __forceinline__ bool interp_prims(const DevModel &m, const S X[4], T pr[8]) {
   if (outside_radially(m, X)) return false;
-  using R = typename std::conditional<F32IDX, float, decltype(vmag(X[0]))>::type;
+  using R = typename std::conditional<F32IDX || std::is_same<S, df>::value, float, double>::type;
   int i, j;
   R di, dj;
   {

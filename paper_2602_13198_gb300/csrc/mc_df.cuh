@@ -108,10 +108,22 @@ __device__ __forceinline__ float to_f(df x) { return __fadd_rn(x.hi, x.lo); }
 // a geodesic scalar in FP32 without an FP64-pipe conversion: narrowed on the integer pipes, or hi + lo
 __device__ __forceinline__ float step_f(double x) { return narrow_f(x); }
 __device__ __forceinline__ float step_f(df x) { return __fadd_rn(x.hi, x.lo); }
-__device__ __forceinline__ double sabs(double x) { return fabs(x); }
-__device__ __forceinline__ df sabs(df x) { return df_abs(x); }
 __device__ __forceinline__ double srcp(double x) { return 1.0 / x; }
 __device__ __forceinline__ df srcp(df x) { return df_rcp(x); }
+// Products, sums and differences that the compiler does not contract: the FP64 geodesic is written out in
+// them and in explicit fused multiply-adds, so that every kernel that inlines it (single-model or batched,
+// a = 0 or general form) rounds alike; the split form's FP32 coefficients read that state.
+__device__ __forceinline__ double smul(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ double sadd(double a, double b) { return __dadd_rn(a, b); }
+__device__ __forceinline__ double ssub(double a, double b) { return __dsub_rn(a, b); }
+__device__ __forceinline__ double stwice(double x) { return __dadd_rn(x, x); }
+__device__ __forceinline__ double shalf(double x) { return __dmul_rn(0.5, x); }
+// a b + c, c - a b, a b - c and a0 b0 + a1 b1
+__device__ __forceinline__ double mad(double a, double b, double c) { return fma(a, b, c); }
+__device__ __forceinline__ double nmad(double a, double b, double c) { return fma(-a, b, c); }
+__device__ __forceinline__ double msub(double a, double b, double c) { return fma(a, b, -c); }
+__device__ __forceinline__ double dot2(double a0, double b0, double a1, double b1) { return fma(a0, b0, __dmul_rn(a1, b1)); }
+
 // ordering of normalised double-float values
 __device__ __forceinline__ bool df_ge(df a, df b) { return a.hi > b.hi || (a.hi == b.hi && a.lo >= b.lo); }
 __device__ __forceinline__ bool df_le(df a, df b) { return a.hi < b.hi || (a.hi == b.hi && a.lo <= b.lo); }
@@ -203,16 +215,14 @@ __device__ __forceinline__ df sdot_mh(df a0, df b0, df c) {
   return dot_end(d);
 }
 
-// Velocity-Verlet updates x + k dl + a dl^2 / 2, k + a dl and k + (a + a') dl / 2, as sums of
-// products for df
-__device__ __forceinline__ double verlet_x(double x, double k, double a, double dl) {
-  return x + k * dl + 0.5f * a * dl * dl;
-}
-__device__ __forceinline__ double verlet_k(double k, double a, double dl) { return k + a * dl; }
-__device__ __forceinline__ double verlet_k2(double k, double a, double a1, double dl) {
-  return k + 0.5f * (a + a1) * dl;
-}
-__device__ __forceinline__ df verlet_x(df x, df k, df a, df dl) {
+// Velocity-Verlet updates x + k dl + a dl^2 / 2, k + a dl and k + (a + a') dl / 2; hd = dl / 2 is read in FP64
+// only, where x + (k + a hd) dl rounds the position once
+__device__ __forceinline__ double half_step(double dl) { return __dmul_rn(0.5, dl); }
+__device__ __forceinline__ double half_step(df) { return 0.0; }
+__device__ __forceinline__ double verlet_x(double x, double k, double a, double dl, double hd) { return fma(fma(a, hd, k), dl, x); }
+__device__ __forceinline__ double verlet_k(double k, double a, double dl) { return fma(a, dl, k); }
+__device__ __forceinline__ double verlet_k2(double k, double a, double a1, double, double hd) { return fma(__dadd_rn(a, a1), hd, k); }
+__device__ __forceinline__ df verlet_x(df x, df k, df a, df dl, double) {
   DotAcc d{x.hi, x.lo};
   dot_add(d, k, dl);
   dot_add(d, df_half(a) * dl, dl);
@@ -223,7 +233,7 @@ __device__ __forceinline__ df verlet_k(df k, df a, df dl) {
   dot_add(d, a, dl);
   return dot_end(d);
 }
-__device__ __forceinline__ df verlet_k2(df k, df a, df a1, df dl) {
+__device__ __forceinline__ df verlet_k2(df k, df a, df a1, df dl, double) {
   DotAcc d{k.hi, k.lo};
   dot_add(d, df_half(a + a1), dl);
   return dot_end(d);
@@ -232,19 +242,44 @@ __device__ __forceinline__ df verlet_k2(df k, df a, df a1, df dl) {
 template <typename S> __device__ __forceinline__ S from_d(double x);
 template <> __device__ __forceinline__ double from_d<double>(double x) { return x; }
 template <> __device__ __forceinline__ df from_d<df>(double x) { return df_from(x); }
-// Terms of the Verlet convergence test sum |k_new - k_old| < tol sum |k_new|: FP64 for double, FP32 for
-// df (the difference of two close df values is exact enough in FP32 once the high parts cancel).
-__device__ __forceinline__ double vdiff(double a, double b) { return fabs(a - b); }
-__device__ __forceinline__ float vdiff(df a, df b) {
-  return fabsf(__fadd_rn(__fsub_rn(a.hi, b.hi), __fsub_rn(a.lo, b.lo)));
+// |x| to 20 bits in FP32, cut from the high word of the double on the integer pipes (0 below the FP32 normal
+// range, 3.4e38 or more above it)
+__device__ __forceinline__ float mag_f(double x) {
+  const int h = __double2hiint(x) & 0x7fffffff;
+  return __int_as_float((min(max(h, 896 << 20), (1151 << 20) - 1) - (896 << 20)) << 3);
 }
-__device__ __forceinline__ double vmag(double a) { return fabs(a); }
-__device__ __forceinline__ float vmag(df a) { return fabsf(a.hi); }
-// a, b >= 0 (sums of magnitudes): compared as bit patterns, off the FP64 pipe
-__device__ __forceinline__ bool below_tol(double a, double tol, float, double b) {
-  return __double_as_longlong(a) < __double_as_longlong(tol * b);
+// Verlet convergence test sum |k_new - k_old| < tol sum |k_new|.  FP64: first in FP32 from the 20-bit
+// magnitudes of the FP64 differences, which decides unless the two sides are within 1% of one another (or
+// leave the FP32 range); only then the FP64 sums are formed, so the outcome is theirs at four instead
+// of eleven FP64 operations.  Sums of magnitudes compare as bit patterns.
+__device__ __forceinline__ bool verlet_converged(const double Kn[4], const double Kp[4], double tol, float tolf) {
+  double d[4];
+  float num = 0.0f, den = 0.0f;
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    d[q] = Kn[q] - Kp[q];
+    num += mag_f(d[q]);
+    den += mag_f(Kn[q]);
+  }
+  const float lim = tolf * den;
+  if (lim > 1e-30f && den < 1e30f) {
+    if (num < 0.99f * lim) return true;
+    if (num > 1.01f * lim) return false;
+  }
+  const double n = fabs(d[0]) + fabs(d[1]) + fabs(d[2]) + fabs(d[3]);
+  const double s = fabs(Kn[0]) + fabs(Kn[1]) + fabs(Kn[2]) + fabs(Kn[3]);
+  return __double_as_longlong(n) < __double_as_longlong(tol * s);
 }
-__device__ __forceinline__ bool below_tol(float a, double, float tolf, float b) { return a < tolf * b; }
+// double-float: in FP32 (the difference of two close df values is exact enough once the high parts cancel)
+__device__ __forceinline__ bool verlet_converged(const df Kn[4], const df Kp[4], double, float tolf) {
+  float num = 0.0f, den = 0.0f;
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    num += fabsf(__fadd_rn(__fsub_rn(Kn[q].hi, Kp[q].hi), __fsub_rn(Kn[q].lo, Kp[q].lo)));
+    den += fabsf(Kn[q].hi);
+  }
+  return num < tolf * den;
+}
 
 // Nearest integer of |x| < 2^22 with FP32 additions only: adding 1.5 * 2^23 leaves the integer in the
 // low mantissa bits (ties to even).  Returns it as a float and, in k, as an int; no conversion

@@ -62,6 +62,39 @@ __device__ __forceinline__ void coefs(const DevModel &m, const GeoT<S> &G, const
   else coefficients64(m, G, X, K, ws, c);
 }
 
+// Geometry of a geodesic step in the geodesic's scalar: the point's Kerr-Schild factors in FP64, the metric
+// with its derivatives in double-float; geo_of gives the metric components for the plasma state.
+template <typename S> struct GeomOf;
+template <> struct GeomOf<double> { using T = Point; };
+template <> struct GeomOf<df> { using T = GeoT<df>; };
+template <bool KERR>
+__device__ __forceinline__ void geom_eval(const DevModel &m, double x1, double x2, Point &G) { point_eval<KERR>(m, x1, x2, G); }
+template <bool KERR>
+__device__ __forceinline__ void geom_eval(const DevModel &m, df x1, df x2, GeoT<df> &G) { metric_eval<true, KERR>(m, x1, x2, G); }
+template <bool KERR>
+__device__ __forceinline__ Geo geo_of(const DevModel &m, const Point &P) {
+  Geo G;
+  metric_of<KERR>(m, P, G);
+  return G;
+}
+template <bool KERR>
+__device__ __forceinline__ const GeoT<df> &geo_of(const DevModel &, const GeoT<df> &G) { return G; }
+template <bool KERR>
+__device__ __forceinline__ void accel(const DevModel &, const GeoT<df> &G, const df k[4], df A[4]) { accel<KERR>(G, k, A); }
+// -k_t and cos(theta): k_t = -k^t + f L with L = k^t + r k^1 - a sin^2 k^phi
+template <bool KERR>
+__device__ __forceinline__ double energy_at_infinity(const Point &G, const double K[4], double &cth) {
+  double L = K[0] + G.r * K[1];
+  if (KERR) L -= G.as2 * K[3];
+  cth = G.c;
+  return K[0] - G.f * L;
+}
+template <bool KERR>
+__device__ __forceinline__ double energy_at_infinity(const GeoT<df> &G, const df K[4], double &cth) {
+  cth = to_d(G.cth);
+  return -(to_d(G.g00) * to_d(K[0]) + to_d(G.g01) * to_d(K[1]) + to_d(G.g03) * to_d(K[3]));
+}
+
 template <bool C32, bool KERR = true>
 static __device__ void init_transport(const DevModel &m, Ph &p) {
   p.x1t = -log(rng_u(p.s, m.seed));
@@ -550,15 +583,16 @@ __device__ __forceinline__ bool at_capture(const DevModel &m, df r) { return df_
 // Binning of a superphoton at the recording sphere (section 3): E_inf = -k_t, log-frequency bin x
 // inclination bin.  The sums are not added here: the bin and w E wait in the state until the warp's
 // flush_record, which adds each bin's share of the warp once.
-template <typename GS, typename S, typename W>
-static __device__ void record(const DevModel &m, const PushIO &io, const GeoT<GS> &G, PhT<S, W> &p) {
-  double E = -(to_d(G.g00) * to_d(p.K[0]) + to_d(G.g01) * to_d(p.K[1]) + to_d(G.g03) * to_d(p.K[3]));
+template <bool KERR, typename GT, typename S, typename W>
+static __device__ void record(const DevModel &m, const PushIO &io, const GT &G, PhT<S, W> &p) {
+  double cth;
+  const double E = energy_at_infinity<KERR>(G, p.K, cth);
   if (!(E > 0.0)) return;
   double nu = E * (kME * kCL * kCL / kHPL);
   double l = log10(nu);
   int ib = (int)floor((l - m.lnu_lo) / m.dlog_bin);
   if (ib < 0 || ib >= m.n_bins) return;
-  double thf = acos(fabs(to_d(G.cth)));
+  double thf = acos(fabs(cth));
   int ii = (int)floor(thf / (0.5 * kPI) * m.n_incl);
   ii = min(max(ii, 0), m.n_incl - 1);
   p.raddr = m.spec + ((int64_t)ii * m.n_bins + ib) * 3;
@@ -692,12 +726,12 @@ __device__ __forceinline__ void absorb_scatter(const DevModel &m, const PushIO &
 
 // Termination tests after a step (recording at r >= r_record, capture, absorption, roulette, step
 // cap); returns the status (0: continue) and writes the log record of a finished superphoton.
-template <typename GS, typename S, typename W>
-__device__ __forceinline__ int terminate(const DevModel &m, const PushIO &io, const GeoT<GS> &G, PhT<S, W> &p,
+template <bool KERR, typename GT, typename S, typename W>
+__device__ __forceinline__ int terminate(const DevModel &m, const PushIO &io, const GT &G, PhT<S, W> &p,
                                          int radius_term, LocalStats &ls) {
   int status = 0;
   if (radius_term == 1) {
-    record(m, io, G, p);
+    record<KERR>(m, io, G, p);
     status = 1;
     ls.rec++;
   } else if (radius_term == 3) {
@@ -724,44 +758,49 @@ __device__ __forceinline__ int terminate(const DevModel &m, const PushIO &io, co
   return status;
 }
 
+// Predictor loop of the Verlet step (reading 2): from (K0, A0) and the point geometry G at x_{n+1}, iterates
+// k_new = K0 + (A0 + A(Kp)) dl / 2 until it moves by less than verlet_tol; Kp enters as the prediction
+// K0 + A0 dl.  Returns k_new and its acceleration, and counts the passes.
+template <bool KERR, typename GT, typename S>
+__device__ __forceinline__ void verlet_loop(const DevModel &m, const GT &G, const S K0[4], const S A0[4], S dl, double hd,
+                                            S Kn[4], S An[4], int &it, bool &conv) {
+  S Kp[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) Kp[q] = verlet_k(K0[q], A0[q], dl);
+  it = 0;
+  conv = false;
+  while (true) {
+    accel<KERR>(m, G, Kp, An);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) Kn[q] = verlet_k2(K0[q], A0[q], An[q], dl, hd);
+    ++it;
+    conv = verlet_converged(Kn, Kp, m.verlet_tol, m.fverlet_tol);
+    if (conv || it >= m.verlet_maxit) break;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) Kp[q] = Kn[q];
+  }
+}
+
 // One geodesic step with absorption, scattering and the termination tests; false when finished.
 template <int PREC, bool KERR = true>
 static __device__ bool step(const DevModel &m, const PushIO &io, PhF<PREC> &p, LocalStats &ls) {
   using S = typename Form<PREC>::S;
   using W = typename Form<PREC>::W;
   const bool scat = m.scatter && p.nsc < m.n_sc_max;
-  S dl = stepsize(m, p.X, p.K);
-  S X0[4], K0[4], Kp[4], An[4];
+  const S dl = stepsize(m, p.X, p.K);
+  const double hd = half_step(dl);
+  S X0[4], K0[4], An[4], Kn[4];
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
     X0[q] = p.X[q];
     K0[q] = p.K[q];
-    p.X[q] = verlet_x(X0[q], K0[q], p.A[q], dl);
-    Kp[q] = verlet_k(K0[q], p.A[q], dl);
+    p.X[q] = verlet_x(X0[q], K0[q], p.A[q], dl, hd);
   }
-  GeoT<S> G;
-  metric_eval<true, KERR>(m, p.X[1], p.X[2], G);
-  int it = 0;
-  bool conv = false;
-  S Kn[4];
-  while (true) {
-    accel<KERR>(G, Kp, An);
-    decltype(vmag(dl)) num = 0, den = 0;
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      Kn[q] = verlet_k2(K0[q], p.A[q], An[q], dl);
-      num += vdiff(Kn[q], Kp[q]);
-      den += vmag(Kn[q]);
-    }
-    ++it;
-#pragma unroll
-    for (int q = 0; q < 4; ++q) Kp[q] = Kn[q];
-    if (below_tol(num, m.verlet_tol, m.fverlet_tol, den)) {
-      conv = true;
-      break;
-    }
-    if (it >= m.verlet_maxit) break;
-  }
+  typename GeomOf<S>::T G;
+  geom_eval<KERR>(m, p.X[1], p.X[2], G);
+  int it;
+  bool conv;
+  verlet_loop<KERR>(m, G, K0, p.A, dl, hd, Kn, An, it, conv);
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
     p.K[q] = Kn[q];
@@ -774,10 +813,10 @@ static __device__ bool step(const DevModel &m, const PushIO &io, PhF<PREC> &p, L
   p.nsteps++;
   ls.steps++;
   CoefT<W> c;
-  coefs<Form<PREC>::C32>(m, G, p.X, p.K, scat, c);
+  coefs<Form<PREC>::C32>(m, geo_of<KERR>(m, G), p.X, p.K, scat, c);
   absorb_scatter(m, io, p, X0, K0, dl, c, scat, ls);
   const int rt = at_record(m, G.r) ? 1 : (at_capture(m, G.r) ? 3 : 0);
-  return terminate(m, io, G, p, rt, ls) == 0;
+  return terminate<KERR>(m, io, G, p, rt, ls) == 0;
 }
 
 // Free-streaming step (both end points outside the grid: no plasma, so tau_a = tau_s = 0 and the
@@ -787,36 +826,17 @@ static __device__ bool step(const DevModel &m, const PushIO &io, PhF<PREC> &p, L
 template <int PREC, bool KERR = true>
 static __device__ int step_free(const DevModel &m, const PushIO &io, PhF<PREC> &p, LocalStats &ls) {
   using S = typename Form<PREC>::S;
-  S dl = stepsize(m, p.X, p.K);
-  S Xn[4], Kp[4], An[4], Kn[4];
+  const S dl = stepsize(m, p.X, p.K);
+  const double hd = half_step(dl);
+  S Xn[4], An[4], Kn[4];
 #pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    Xn[q] = verlet_x(p.X[q], p.K[q], p.A[q], dl);
-    Kp[q] = verlet_k(p.K[q], p.A[q], dl);
-  }
+  for (int q = 0; q < 4; ++q) Xn[q] = verlet_x(p.X[q], p.K[q], p.A[q], dl, hd);
   if (in_grid(m, Xn)) return 2;
-  GeoT<S> G;
-  metric_eval<true, KERR>(m, Xn[1], Xn[2], G);
-  int it = 0;
-  bool conv = false;
-  while (true) {
-    accel<KERR>(G, Kp, An);
-    decltype(vmag(dl)) num = 0, den = 0;
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      Kn[q] = verlet_k2(p.K[q], p.A[q], An[q], dl);
-      num += vdiff(Kn[q], Kp[q]);
-      den += vmag(Kn[q]);
-    }
-    ++it;
-#pragma unroll
-    for (int q = 0; q < 4; ++q) Kp[q] = Kn[q];
-    if (below_tol(num, m.verlet_tol, m.fverlet_tol, den)) {
-      conv = true;
-      break;
-    }
-    if (it >= m.verlet_maxit) break;
-  }
+  typename GeomOf<S>::T G;
+  geom_eval<KERR>(m, Xn[1], Xn[2], G);
+  int it;
+  bool conv;
+  verlet_loop<KERR>(m, G, p.K, p.A, dl, hd, Kn, An, it, conv);
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
     p.X[q] = Xn[q];
@@ -830,7 +850,7 @@ static __device__ int step_free(const DevModel &m, const PushIO &io, PhF<PREC> &
   p.ana = 0;
   p.ans = 0;
   const int rt = at_record(m, G.r) ? 1 : (at_capture(m, G.r) ? 3 : 0);
-  return terminate(m, io, G, p, rt, ls) ? 1 : 0;
+  return terminate<KERR>(m, io, G, p, rt, ls) ? 1 : 0;
 }
 
 __device__ __forceinline__ unsigned long long warp_sum(unsigned long long v) {
@@ -925,37 +945,20 @@ struct SurCarry {
 
 template <typename S, typename W>
 static __device__ void step_sur_a(const DevModel &m, PhT<S, W> &p, SurCarry<S> &sc, LocalStats &ls) {
-  S dl = stepsize(m, p.X, p.K);
-  S Kp[4], An[4], Kn[4];
+  const S dl = stepsize(m, p.X, p.K);
+  const double hd = half_step(dl);
+  S An[4], Kn[4];
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
     sc.X0[q] = p.X[q];
     sc.K0[q] = p.K[q];
-    p.X[q] = verlet_x(sc.X0[q], sc.K0[q], p.A[q], dl);
-    Kp[q] = verlet_k(sc.K0[q], p.A[q], dl);
+    p.X[q] = verlet_x(sc.X0[q], sc.K0[q], p.A[q], dl, hd);
   }
-  GeoT<S> G;
-  metric_eval<true>(m, p.X[1], p.X[2], G);
-  int it = 0;
-  bool conv = false;
-  while (true) {
-    accel(G, Kp, An);
-    decltype(vmag(dl)) num = 0, den = 0;
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      Kn[q] = verlet_k2(sc.K0[q], p.A[q], An[q], dl);
-      num += vdiff(Kn[q], Kp[q]);
-      den += vmag(Kn[q]);
-    }
-    ++it;
-#pragma unroll
-    for (int q = 0; q < 4; ++q) Kp[q] = Kn[q];
-    if (below_tol(num, m.verlet_tol, m.fverlet_tol, den)) {
-      conv = true;
-      break;
-    }
-    if (it >= m.verlet_maxit) break;
-  }
+  typename GeomOf<S>::T G;
+  geom_eval<true>(m, p.X[1], p.X[2], G);
+  int it;
+  bool conv;
+  verlet_loop<true>(m, G, sc.K0, p.A, dl, hd, Kn, An, it, conv);
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
     p.K[q] = Kn[q];
@@ -970,7 +973,7 @@ static __device__ void step_sur_a(const DevModel &m, PhT<S, W> &p, SurCarry<S> &
   sc.dl = dl;
   // only the radius tests cross the network evaluation (the metric is re-evaluated to record)
   sc.term = at_record(m, G.r) ? 1 : (at_capture(m, G.r) ? 3 : 0);
-  coefficients32_a(m, G, p.X, p.K, sc.a);
+  coefficients32_a(m, geo_of<true>(m, G), p.X, p.K, sc.a);
 }
 
 template <int PREC>
@@ -981,13 +984,9 @@ static __device__ bool step_sur_b(const DevModel &m, const PushIO &io, PhF<PREC>
   CoefT<W> c;
   coefficients32_b(m, sc.a, out, scat, c);
   absorb_scatter(m, io, p, sc.X0, sc.K0, sc.dl, c, scat, ls);
-  if (sc.term == 1) {
-    GeoT<typename Form<PREC>::S> G;
-    metric_eval<false>(m, p.X[1], p.X[2], G);
-    return terminate(m, io, G, p, 1, ls) == 0;
-  }
-  const Geo Gd{};   // not read: recording needs the metric only when sc.term == 1
-  return terminate(m, io, Gd, p, sc.term, ls) == 0;
+  typename GeomOf<typename Form<PREC>::S>::T G;   // read only by the recording (sc.term == 1)
+  if (sc.term == 1) geom_eval<true>(m, p.X[1], p.X[2], G);
+  return terminate<true>(m, io, G, p, sc.term, ls) == 0;
 }
 
 }  // namespace mcgb
