@@ -597,7 +597,7 @@ static int transport(mc_ctx *c, int64_t u0, int64_t u1, const int64_t *uid_list_
   int occ_sur = 1;
   if (use_sur) {
     sv = surrogate_view(c);
-    occ_sur = std::max(1, std::min(4, push_sur_max_blocks_per_sm(prec, sur_block, sur_smem)));
+    occ_sur = std::max(1, std::min(4, push_sur_max_blocks_per_sm(prec, sur_block, sur_smem, m.a != 0.0 ? 1 : 0)));
     if (c->p.ctas_per_sm > 0) occ_sur = std::min(occ_sur, (int)c->p.ctas_per_sm);
     CU(cudaMemsetAsync(c->sur_err, 0, sizeof(unsigned int), st));
   }

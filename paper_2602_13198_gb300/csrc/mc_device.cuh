@@ -762,9 +762,9 @@ __device__ __forceinline__ void metric_of(const DevModel &m, const Point &P, Geo
 // About 55 multiply-adds; contracting the metric's derivatives (14 of them, with 13 components) took
 // about 200 operations and kept all of them live across the predictor loop.  The FP64 pipe bounds these kernels
 // (one warp instruction per 64 cycles on each SM partition), so the count is the time: one shard of the 3-D
-// snapshot went from 539 to 442 ms in FP64 and from 401 to 303 ms in the split form with the network.  KERR = false leaves out the
-// terms that are exactly zero at a = 0 and nothing else, so that the two forms agree bit for bit there (a
-// batch runs every model in the general form).
+// snapshot went from 539 to 442 ms in FP64 and from 401 to 303 ms in the split form with the network.
+// KERR = false leaves out the terms that are exactly zero at a = 0 and nothing else, so that the two forms agree
+// bit for bit there (a batch runs every model in the general form).
 template <bool KERR = true>
 __device__ __forceinline__ void accel(const DevModel &m, const Point &G, const double k[4], double A[4]) {
   const double k1 = k[1], kp = k[3];
@@ -814,19 +814,26 @@ __device__ __forceinline__ void accel(const DevModel &m, const Point &G, const d
 
 // Step size (reading; the paper gives none): each internal coordinate moves at most eps_geo of
 // its scale (1 for ln r and phi, the distance to the nearer pole for x2).
-template <typename S = double>
-__device__ __forceinline__ S stepsize(const DevModel &m, const S X[4], const S K[4]) {
-  // 1 / (1/d1 + 1/d2 + 1/d3) with d1 = eps/|k1|, d2 = eps x2n/|k2|, d3 = eps/|k3|
-  // = eps x2n / ((|k1| + |k3|) x2n + |k2|): one reciprocal
-  const double x2n = dmin_nn(fabs(X[2]), fabs(__dsub_rn(1.0, X[2])));
-  const double den = fma(__dadd_rn(fabs(K[1]), fabs(K[3])), x2n, __dadd_rn(fabs(K[2]), 1e-40));
-  return __dmul_rn(__dmul_rn(m.eps_geo, x2n), rcp_n(den));
+//   1 / (1/d1 + 1/d2 + 1/d3) with d1 = eps/(|k1|+S), d2 = eps x2n/(|k2|+S), d3 = eps/(|k3|+S)
+//   = eps x2n / ((|k1| + |k3|) x2n + |k2|): one division, or one reciprocal with the point form.
+template <bool POINT>
+__device__ __forceinline__ double stepsize(const DevModel &m, const double X[4], const double K[4]) {
+  if constexpr (POINT) {
+    const double x2n = dmin_nn(fabs(X[2]), fabs(__dsub_rn(1.0, X[2])));
+    const double den = fma(__dadd_rn(fabs(K[1]), fabs(K[3])), x2n, __dadd_rn(fabs(K[2]), 1e-40));
+    return __dmul_rn(__dmul_rn(m.eps_geo, x2n), rcp_n(den));
+  } else {
+    const double SMALL = 1e-40;
+    double x2n = dmin_nn(fabs(X[2]), fabs(1.0 - X[2]));
+    double den = ((fabs(K[1]) + SMALL) + (fabs(K[3]) + SMALL)) * x2n + (fabs(K[2]) + SMALL);
+    return m.eps_geo * x2n / den;
+  }
 }
 
 // Double-float step size: the same rule in double-float, so that the steps land where the FP64
 // path's do (an FP32 step length would move every step end along the path by ~1e-7).
-template <>
-__device__ __forceinline__ df stepsize<df>(const DevModel &m, const df X[4], const df K[4]) {
+template <bool>
+__device__ __forceinline__ df stepsize(const DevModel &m, const df X[4], const df K[4]) {
   const df a = df_abs(X[2]), b = df_abs(1.0f - X[2]);
   const df x2n = df_le(a, b) ? a : b;
   const df den = ((df_abs(K[1]) + df_abs(K[3])) * x2n + df_abs(K[2])) + 1e-30f;

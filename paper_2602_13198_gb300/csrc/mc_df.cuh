@@ -215,24 +215,40 @@ __device__ __forceinline__ df sdot_mh(df a0, df b0, df c) {
   return dot_end(d);
 }
 
-// Velocity-Verlet updates x + k dl + a dl^2 / 2, k + a dl and k + (a + a') dl / 2; hd = dl / 2 is read in FP64
-// only, where x + (k + a hd) dl rounds the position once
+// Velocity-Verlet updates x + k dl + a dl^2 / 2, k + a dl and k + (a + a') dl / 2.  FP64 with POINT: explicit fused
+// multiply-adds with hd = dl / 2, the position rounded once (x + (k + a hd) dl); without it the plain
+// expressions, which belong to the component form of the geometry.
 __device__ __forceinline__ double half_step(double dl) { return __dmul_rn(0.5, dl); }
 __device__ __forceinline__ double half_step(df) { return 0.0; }
-__device__ __forceinline__ double verlet_x(double x, double k, double a, double dl, double hd) { return fma(fma(a, hd, k), dl, x); }
-__device__ __forceinline__ double verlet_k(double k, double a, double dl) { return fma(a, dl, k); }
-__device__ __forceinline__ double verlet_k2(double k, double a, double a1, double, double hd) { return fma(__dadd_rn(a, a1), hd, k); }
+template <bool POINT>
+__device__ __forceinline__ double verlet_x(double x, double k, double a, double dl, double hd) {
+  if constexpr (POINT) return fma(fma(a, hd, k), dl, x);
+  else return x + k * dl + 0.5f * a * dl * dl;
+}
+template <bool POINT>
+__device__ __forceinline__ double verlet_k(double k, double a, double dl) {
+  if constexpr (POINT) return fma(a, dl, k);
+  else return k + a * dl;
+}
+template <bool POINT>
+__device__ __forceinline__ double verlet_k2(double k, double a, double a1, double dl, double hd) {
+  if constexpr (POINT) return fma(__dadd_rn(a, a1), hd, k);
+  else return k + 0.5f * (a + a1) * dl;
+}
+template <bool>
 __device__ __forceinline__ df verlet_x(df x, df k, df a, df dl, double) {
   DotAcc d{x.hi, x.lo};
   dot_add(d, k, dl);
   dot_add(d, df_half(a) * dl, dl);
   return dot_end(d);
 }
+template <bool>
 __device__ __forceinline__ df verlet_k(df k, df a, df dl) {
   DotAcc d{k.hi, k.lo};
   dot_add(d, a, dl);
   return dot_end(d);
 }
+template <bool>
 __device__ __forceinline__ df verlet_k2(df k, df a, df a1, df dl, double) {
   DotAcc d{k.hi, k.lo};
   dot_add(d, df_half(a + a1), dl);

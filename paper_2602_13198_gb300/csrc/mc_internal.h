@@ -101,7 +101,7 @@ void launch_init(const DevModel &m, const InitIO &io, int prec, int grid, int bl
 // phase 0: superphotons inside the radial extent of the grid; 1: outside it
 void launch_push(const DevModel &m, const PushIO &io, int prec, int phase, int grid, int block, cudaStream_t st);
 // in-grid push with the coefficient network (mixed or split form; 128-thread row groups)
-int push_sur_max_blocks_per_sm(int prec, int block, int smem);
+int push_sur_max_blocks_per_sm(int prec, int block, int smem, int kerr);
 void launch_push_sur(const DevModel &m, const PushIO &io, const SurrogateView &sv, int prec, int grid, int smem,
                      cudaStream_t st);
 

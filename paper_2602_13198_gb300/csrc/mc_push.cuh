@@ -62,25 +62,29 @@ __device__ __forceinline__ void coefs(const DevModel &m, const GeoT<S> &G, const
   else coefficients64(m, G, X, K, ws, c);
 }
 
-// Geometry of a geodesic step in the geodesic's scalar: the point's Kerr-Schild factors in FP64, the metric
-// with its derivatives in double-float; geo_of gives the metric components for the plasma state.
-template <typename S> struct GeomOf;
-template <> struct GeomOf<double> { using T = Point; };
-template <> struct GeomOf<df> { using T = GeoT<df>; };
+// Geometry of a geodesic step: POINT, the point's Kerr-Schild factors (FP64); otherwise the metric's components
+// and derivatives, in double-float or, in the split form's in-grid steps where a = 0 can occur (single models
+// with a = 0, and batches), in FP64: that form narrows the components to FP32 by truncation, and
+// g_t1 = f r = 2 M exactly at a = 0, so a last-bit difference in FP64 is a whole FP32 step (6e-8) in the
+// coefficients, which moved some spectra by 4e-9.
+template <int PREC, bool KERR, bool BATCH>
+constexpr bool kPointForm = PREC == 0 || (PREC == 2 && KERR && !BATCH);
+template <bool POINT, typename S> struct GeomOf { using T = GeoT<S>; };
+template <> struct GeomOf<true, double> { using T = Point; };
 template <bool KERR>
 __device__ __forceinline__ void geom_eval(const DevModel &m, double x1, double x2, Point &G) { point_eval<KERR>(m, x1, x2, G); }
-template <bool KERR>
-__device__ __forceinline__ void geom_eval(const DevModel &m, df x1, df x2, GeoT<df> &G) { metric_eval<true, KERR>(m, x1, x2, G); }
+template <bool KERR, typename S>
+__device__ __forceinline__ void geom_eval(const DevModel &m, S x1, S x2, GeoT<S> &G) { metric_eval<true, KERR>(m, x1, x2, G); }
+template <bool KERR, typename S>
+__device__ __forceinline__ void accel(const DevModel &, const GeoT<S> &G, const S k[4], S A[4]) { accel<KERR>(G, k, A); }
 template <bool KERR>
 __device__ __forceinline__ Geo geo_of(const DevModel &m, const Point &P) {
   Geo G;
   metric_of<KERR>(m, P, G);
   return G;
 }
-template <bool KERR>
-__device__ __forceinline__ const GeoT<df> &geo_of(const DevModel &, const GeoT<df> &G) { return G; }
-template <bool KERR>
-__device__ __forceinline__ void accel(const DevModel &, const GeoT<df> &G, const df k[4], df A[4]) { accel<KERR>(G, k, A); }
+template <bool KERR, typename S>
+__device__ __forceinline__ const GeoT<S> &geo_of(const DevModel &, const GeoT<S> &G) { return G; }
 // -k_t and cos(theta): k_t = -k^t + f L with L = k^t + r k^1 - a sin^2 k^phi
 template <bool KERR>
 __device__ __forceinline__ double energy_at_infinity(const Point &G, const double K[4], double &cth) {
@@ -89,8 +93,8 @@ __device__ __forceinline__ double energy_at_infinity(const Point &G, const doubl
   cth = G.c;
   return K[0] - G.f * L;
 }
-template <bool KERR>
-__device__ __forceinline__ double energy_at_infinity(const GeoT<df> &G, const df K[4], double &cth) {
+template <bool KERR, typename S>
+__device__ __forceinline__ double energy_at_infinity(const GeoT<S> &G, const S K[4], double &cth) {
   cth = to_d(G.cth);
   return -(to_d(G.g00) * to_d(K[0]) + to_d(G.g01) * to_d(K[1]) + to_d(G.g03) * to_d(K[3]));
 }
@@ -758,21 +762,21 @@ __device__ __forceinline__ int terminate(const DevModel &m, const PushIO &io, co
   return status;
 }
 
-// Predictor loop of the Verlet step (reading 2): from (K0, A0) and the point geometry G at x_{n+1}, iterates
+// Predictor loop of the Verlet step (reading 2): from (K0, A0) and the geometry G at x_{n+1}, iterates
 // k_new = K0 + (A0 + A(Kp)) dl / 2 until it moves by less than verlet_tol; Kp enters as the prediction
 // K0 + A0 dl.  Returns k_new and its acceleration, and counts the passes.
-template <bool KERR, typename GT, typename S>
+template <bool KERR, bool POINT, typename GT, typename S>
 __device__ __forceinline__ void verlet_loop(const DevModel &m, const GT &G, const S K0[4], const S A0[4], S dl, double hd,
                                             S Kn[4], S An[4], int &it, bool &conv) {
   S Kp[4];
 #pragma unroll
-  for (int q = 0; q < 4; ++q) Kp[q] = verlet_k(K0[q], A0[q], dl);
+  for (int q = 0; q < 4; ++q) Kp[q] = verlet_k<POINT>(K0[q], A0[q], dl);
   it = 0;
   conv = false;
   while (true) {
     accel<KERR>(m, G, Kp, An);
 #pragma unroll
-    for (int q = 0; q < 4; ++q) Kn[q] = verlet_k2(K0[q], A0[q], An[q], dl, hd);
+    for (int q = 0; q < 4; ++q) Kn[q] = verlet_k2<POINT>(K0[q], A0[q], An[q], dl, hd);
     ++it;
     conv = verlet_converged(Kn, Kp, m.verlet_tol, m.fverlet_tol);
     if (conv || it >= m.verlet_maxit) break;
@@ -782,25 +786,26 @@ __device__ __forceinline__ void verlet_loop(const DevModel &m, const GT &G, cons
 }
 
 // One geodesic step with absorption, scattering and the termination tests; false when finished.
-template <int PREC, bool KERR = true>
+template <int PREC, bool KERR, bool BATCH>
 static __device__ bool step(const DevModel &m, const PushIO &io, PhF<PREC> &p, LocalStats &ls) {
   using S = typename Form<PREC>::S;
   using W = typename Form<PREC>::W;
+  constexpr bool POINT = kPointForm<PREC, KERR, BATCH>;
   const bool scat = m.scatter && p.nsc < m.n_sc_max;
-  const S dl = stepsize(m, p.X, p.K);
+  const S dl = stepsize<POINT>(m, p.X, p.K);
   const double hd = half_step(dl);
   S X0[4], K0[4], An[4], Kn[4];
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
     X0[q] = p.X[q];
     K0[q] = p.K[q];
-    p.X[q] = verlet_x(X0[q], K0[q], p.A[q], dl, hd);
+    p.X[q] = verlet_x<POINT>(X0[q], K0[q], p.A[q], dl, hd);
   }
-  typename GeomOf<S>::T G;
+  typename GeomOf<POINT, S>::T G;
   geom_eval<KERR>(m, p.X[1], p.X[2], G);
   int it;
   bool conv;
-  verlet_loop<KERR>(m, G, K0, p.A, dl, hd, Kn, An, it, conv);
+  verlet_loop<KERR, POINT>(m, G, K0, p.A, dl, hd, Kn, An, it, conv);
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
     p.K[q] = Kn[q];
@@ -826,17 +831,17 @@ static __device__ bool step(const DevModel &m, const PushIO &io, PhF<PREC> &p, L
 template <int PREC, bool KERR = true>
 static __device__ int step_free(const DevModel &m, const PushIO &io, PhF<PREC> &p, LocalStats &ls) {
   using S = typename Form<PREC>::S;
-  const S dl = stepsize(m, p.X, p.K);
+  const S dl = stepsize<true>(m, p.X, p.K);
   const double hd = half_step(dl);
   S Xn[4], An[4], Kn[4];
 #pragma unroll
-  for (int q = 0; q < 4; ++q) Xn[q] = verlet_x(p.X[q], p.K[q], p.A[q], dl, hd);
+  for (int q = 0; q < 4; ++q) Xn[q] = verlet_x<true>(p.X[q], p.K[q], p.A[q], dl, hd);
   if (in_grid(m, Xn)) return 2;
-  typename GeomOf<S>::T G;
+  typename GeomOf<true, S>::T G;
   geom_eval<KERR>(m, Xn[1], Xn[2], G);
   int it;
   bool conv;
-  verlet_loop<KERR>(m, G, p.K, p.A, dl, hd, Kn, An, it, conv);
+  verlet_loop<KERR, true>(m, G, p.K, p.A, dl, hd, Kn, An, it, conv);
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
     p.X[q] = Xn[q];
@@ -943,22 +948,22 @@ struct SurCarry {
   CoefA a;
 };
 
-template <typename S, typename W>
+template <bool POINT, typename S, typename W>
 static __device__ void step_sur_a(const DevModel &m, PhT<S, W> &p, SurCarry<S> &sc, LocalStats &ls) {
-  const S dl = stepsize(m, p.X, p.K);
+  const S dl = stepsize<POINT>(m, p.X, p.K);
   const double hd = half_step(dl);
   S An[4], Kn[4];
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
     sc.X0[q] = p.X[q];
     sc.K0[q] = p.K[q];
-    p.X[q] = verlet_x(sc.X0[q], sc.K0[q], p.A[q], dl, hd);
+    p.X[q] = verlet_x<POINT>(sc.X0[q], sc.K0[q], p.A[q], dl, hd);
   }
-  typename GeomOf<S>::T G;
+  typename GeomOf<POINT, S>::T G;
   geom_eval<true>(m, p.X[1], p.X[2], G);
   int it;
   bool conv;
-  verlet_loop<true>(m, G, sc.K0, p.A, dl, hd, Kn, An, it, conv);
+  verlet_loop<true, POINT>(m, G, sc.K0, p.A, dl, hd, Kn, An, it, conv);
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
     p.K[q] = Kn[q];
@@ -976,7 +981,7 @@ static __device__ void step_sur_a(const DevModel &m, PhT<S, W> &p, SurCarry<S> &
   coefficients32_a(m, geo_of<true>(m, G), p.X, p.K, sc.a);
 }
 
-template <int PREC>
+template <int PREC, bool POINT>
 static __device__ bool step_sur_b(const DevModel &m, const PushIO &io, PhF<PREC> &p,
                                   const SurCarry<typename Form<PREC>::S> &sc, const float out[3], LocalStats &ls) {
   using W = typename Form<PREC>::W;
@@ -984,7 +989,7 @@ static __device__ bool step_sur_b(const DevModel &m, const PushIO &io, PhF<PREC>
   CoefT<W> c;
   coefficients32_b(m, sc.a, out, scat, c);
   absorb_scatter(m, io, p, sc.X0, sc.K0, sc.dl, c, scat, ls);
-  typename GeomOf<typename Form<PREC>::S>::T G;   // read only by the recording (sc.term == 1)
+  typename GeomOf<POINT, typename Form<PREC>::S>::T G;   // read only by the recording (sc.term == 1)
   if (sc.term == 1) geom_eval<true>(m, p.X[1], p.X[2], G);
   return terminate<true>(m, io, G, p, sc.term, ls) == 0;
 }

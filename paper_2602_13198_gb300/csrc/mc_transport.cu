@@ -96,7 +96,7 @@ __device__ __forceinline__ void push_body(const DevModel &m, const PushIO &io) {
     if (live) {
       bool handoff;
       if (PHASE == 0) {
-        live = step<PREC, KERR>(m, io, p, ls);
+        live = step<PREC, KERR, false>(m, io, p, ls);
         handoff = live && !in_grid(m, p.X);
       } else {
         int r = step_free<PREC, KERR>(m, io, p, ls);
@@ -148,7 +148,7 @@ __global__ void __launch_bounds__(128, MC_SPLIT_MINB) k_push_split(DevModel m, P
 // Persistent in-grid push with the network.  Each 128-thread row group reaches its tensor-core
 // evaluation once per iteration (idle lanes contribute a zero row) and leaves the loop as a whole;
 // the CTA's groups iterate independently and meet again only at the teardown.
-template <int PREC>
+template <int PREC, bool KERR>
 __global__ void __launch_bounds__(128 * kTcGroupsMax) k_push_sur(DevModel m, PushIO io, SurrogateView sv) {
   extern __shared__ __align__(128) unsigned char smem_sur[];
   TcMlp T;
@@ -188,14 +188,14 @@ __global__ void __launch_bounds__(128 * kTcGroupsMax) k_push_sur(DevModel m, Pus
     }
     float in[3] = {0.0f, 0.0f, 0.0f}, out[3];
     if (live) {
-      step_sur_a(m, p, sc, ls);
+      step_sur_a<kPointForm<PREC, KERR, false>>(m, p, sc, ls);
       in[0] = sc.a.in[0];
       in[1] = sc.a.in[1];
       in[2] = sc.a.in[2];
     }
     tc_mlp_eval(T, in, out);
     if (live) {
-      live = step_sur_b<PREC>(m, io, p, sc, out, ls);
+      live = step_sur_b<PREC, kPointForm<PREC, KERR, false>>(m, io, p, sc, out, ls);
       if (live && !in_grid(m, p.X)) {
         save_ph(io.pool, slot, p);
         unsigned long long o = atomicAdd(io.cnt + io.out_counter, 1ull);
@@ -209,13 +209,14 @@ __global__ void __launch_bounds__(128 * kTcGroupsMax) k_push_sur(DevModel m, Pus
   flush_stats(ls, io.cnt);
 }
 
-static const void *sur_kernel(int prec) {
-  return prec == 2 ? (const void *)k_push_sur<2> : (const void *)k_push_sur<1>;
+static const void *sur_kernel(int prec, bool kerr) {
+  if (prec == 2) return kerr ? (const void *)k_push_sur<2, true> : (const void *)k_push_sur<2, false>;
+  return (const void *)k_push_sur<1, true>;   // double-float: the general form covers a = 0 bit for bit
 }
 
-int push_sur_max_blocks_per_sm(int prec, int block, int smem) {
+int push_sur_max_blocks_per_sm(int prec, int block, int smem, int kerr) {
   int n = 0;
-  const void *k = sur_kernel(prec);
+  const void *k = sur_kernel(prec, kerr != 0);
   cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, block, smem);
@@ -224,8 +225,8 @@ int push_sur_max_blocks_per_sm(int prec, int block, int smem) {
 
 void launch_push_sur(const DevModel &m, const PushIO &io, const SurrogateView &sv, int prec, int grid, int smem,
                      cudaStream_t st) {
-  if (prec == 2) k_push_sur<2><<<grid, 128 * kTcGroupsMax, smem, st>>>(m, io, sv);
-  else k_push_sur<1><<<grid, 128 * kTcGroupsMax, smem, st>>>(m, io, sv);
+  void *args[] = {(void *)&m, (void *)&io, (void *)&sv};
+  cudaLaunchKernel(sur_kernel(prec, m.a != 0.0), dim3(grid), dim3(128 * kTcGroupsMax), args, smem, st);
 }
 
 // Kernel of one launch configuration: precision form, phase and spin (general Kerr, or a = 0).
