@@ -203,6 +203,7 @@ DevModel make_model(const mc_ctx *c) {
   m.zbq = c->zbq;
   m.zbnt = c->zbnt;
   m.lnF = c->lnF;
+  m.lnFc = c->lnFc;
   m.nF = c->nF;
   m.lnK2 = c->lnK2;
   m.nK2 = c->nK2;
@@ -293,6 +294,7 @@ int mc_init_model(mc_ctx **out, const mc_model_params *p) {
   c->nF = (int)std::floor((kFLnK1 - kFLnK0) / kFStep + 0.5) + 1;
   c->nK2 = (int)std::floor((kK2LnT1 - kK2LnT0) / kK2Step + 0.5) + 1;
   c->lnF = (double *)dev_alloc(c, sizeof(double) * c->nF);
+  c->lnFc = (double *)dev_alloc(c, sizeof(double) * 4 * (c->nF - 1));
   c->lnK2 = (double *)dev_alloc(c, sizeof(double) * c->nK2);
   c->lnK2f = (float *)dev_alloc(c, sizeof(float) * c->nK2);
   c->hotf = (float *)dev_alloc(c, sizeof(float) * kHotNT * kHotNE);
@@ -307,7 +309,7 @@ int mc_init_model(mc_ctx **out, const mc_model_params *p) {
   c->lnw = (double *)dev_alloc(c, sizeof(double) * p->n_nu);
   c->winv = (double *)dev_alloc(c, sizeof(double) * p->n_nu);
   c->bad = (int *)dev_alloc(c, sizeof(int));
-  if (!c->lnF || !c->lnK2 || !c->hot || !c->gl || !c->cnt || !c->total_dev || !c->spec || !c->lnw || !c->winv || !c->bad) {
+  if (!c->lnF || !c->lnFc || !c->lnK2 || !c->hot || !c->gl || !c->cnt || !c->total_dev || !c->spec || !c->lnw || !c->winv || !c->bad) {
     mc_free(c);
     return fail(nullptr, MC_ERR_OOM, "device allocation failed");
   }
@@ -356,7 +358,7 @@ int mc_init_model(mc_ctx **out, const mc_model_params *p) {
     launch_kappa_tables(p->kappa, c->kapF, c->kapJ, c->kapA, c->kapI, c->kapH, c->gl + 256, 0);
   }
   DevModel m = make_model(c);
-  launch_tables(m, c->lnF, c->lnK2, c->hot, c->gl, c->gl + 128, c->gl + 256, 0);
+  launch_tables(m, c->lnF, c->lnFc, c->lnK2, c->hot, c->gl, c->gl + 128, c->gl + 256, 0);
   if (!c->lnK2f || !c->hotf) {
     mc_free(c);
     return fail(nullptr, MC_ERR_OOM, "device allocation failed");

@@ -82,7 +82,8 @@ __device__ __forceinline__ double dmax_nn(double a, double b) {
 // host in extended precision (ftab_host).  Measured on GB300, in FP64-pipe FMA-equivalents per call:
 // exp 10.9 against 15.1 for CUDA's, log 14.8 against 28.7.  Checked against CUDA's functions by
 // mc_selftest_math.
-constexpr int kFtExp = 0, kFtInvC = 32, kFtLogHi = 160, kFtLogLo = 288, kFtSin = 416, kFtCos = 480, kFtN = 544;
+constexpr int kFtExp = 0, kFtInvC = 32, kFtLogHi = 160, kFtLogLo = 288, kFtSin = 416, kFtCos = 480, kFtExpQ = 544,
+              kFtN = 800;
 void ftab_host(double *t);
 
 // e^x = 2^m 2^(j/32) e^r with x = (32 m + j) ln2/32 + r, |r| <= ln2/64 (n = 32 m + j by the 1.5 * 2^52
@@ -105,6 +106,24 @@ __device__ __forceinline__ double exp_t(const double *T, double x) {
   const double tj = __ldg(T + kFtExp + (n & 31));
   const double y = fma(tj, pm1, tj);
   return __hiloint2double(__double2hiint(y) + ((n >> 5) << 20), __double2loint(y));
+}
+
+// e^x from 2^(j/256): |r| <= ln2/512, so the series stops at r^4 (truncation below 4e-17) and the call takes 9
+// FP64 operations instead of 11; the 2 KB of table stay in L1.
+__device__ __forceinline__ double exp_q(const double *T, double x) {
+  if (!((__double_as_longlong(x) & 0x7fffffffffffffffLL) < 0x4086200000000000LL)) return exp(x);   // |x| < 708
+  const double sh = 6755399441055744.0;
+  const double t = fma(x, 369.3299304675746, sh);   // 256 / ln2
+  const int n = __double2loint(t);
+  const double nd = t - sh;
+  double r = fma(nd, -0.00270760617331689, x);
+  r = fma(nd, -7.453964567463233e-13, r);
+  double q = fma(r, 1.0 / 24.0, 1.0 / 6.0);
+  q = fma(q, r, 0.5);
+  const double pm1 = fma(q, r * r, r);
+  const double tj = __ldg(T + kFtExpQ + (n & 255));
+  const double y = fma(tj, pm1, tj);
+  return __hiloint2double(__double2hiint(y) + ((n >> 8) << 20), __double2loint(y));
 }
 
 // e^x - 1: for |x| < 1/4 its Taylor series to x^12 (truncation below 1e-17 relative), by Horner in
@@ -249,6 +268,7 @@ struct DevModel {
   const float *prim32x;   // FP32 primitives for the FP32 coefficient path (the grid or a copy), or NULL
   // tables
   const double *lnF;      // angle integral
+  const double *lnFc;     // its cubics per cell (see F_cells)
   int nF;
   const double *lnK2;
   int nK2;

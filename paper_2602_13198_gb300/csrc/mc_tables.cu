@@ -10,6 +10,8 @@
 // Per run: zone volumes and emission prefactors, the weight table w(nu_j) (eq. weight_calc, a
 // deterministic two-pass reduction over zones), expected zone counts, their stochastic rounding
 // with the zone's Philox stream, and an exclusive scan giving each zone's first superphoton uid.
+#include <cstring>
+
 #include "mc_internal.h"
 
 namespace mcgb {
@@ -65,9 +67,26 @@ __global__ void k_table_hot(double *hot, const double *gsx, const double *gsw, c
   hot[idx] = log(num / den);
 }
 
-void launch_tables(const DevModel &m, double *lnF, double *lnK2, double *hot, const double *gl_ang, const double *gl_s,
+// The 4-point Lagrange cubics of cubic_table as polynomials in the offset t from each cell's left node: cell c
+// of the n - 1 cells takes nodes i - 1 .. i + 2 with i = c kept within [1, n - 3].
+__global__ void k_cubic_cells(const double *y, int n, double *cell) {
+  const int c = blockIdx.x * blockDim.x + threadIdx.x;
+  if (c >= n - 1) return;
+  const int i = max(1, min(c, n - 3));
+  const double y0 = y[i - 1], y1 = y[i], y2 = y[i + 1], y3 = y[i + 2];
+  const double a1 = y2 - y0 / 3.0 - 0.5 * y1 - y3 / 6.0, a2 = 0.5 * (y0 + y2) - y1,
+               a3 = (y3 - y0) / 6.0 + 0.5 * (y1 - y2);
+  const double d = c - i;   // offset from node i: u = t + d
+  cell[4 * c] = y1 + d * (a1 + d * (a2 + d * a3));
+  cell[4 * c + 1] = a1 + d * (2.0 * a2 + 3.0 * d * a3);
+  cell[4 * c + 2] = a2 + 3.0 * d * a3;
+  cell[4 * c + 3] = a3;
+}
+
+void launch_tables(const DevModel &m, double *lnF, double *lnFc, double *lnK2, double *hot, const double *gl_ang, const double *gl_s,
                    const double *gl_mu, cudaStream_t st) {
   k_table_F<<<(m.nF + 127) / 128, 128, 0, st>>>(lnF, m.nF, gl_ang, gl_ang + 64);
+  k_cubic_cells<<<(m.nF + 126) / 128, 128, 0, st>>>(lnF, m.nF, lnFc);
   k_table_K2<<<(m.nK2 + 127) / 128, 128, 0, st>>>(lnK2, m.nK2);
   k_table_hot<<<(kHotNT * kHotNE + 127) / 128, 128, 0, st>>>(hot, gl_s, gl_s + 64, gl_mu, gl_mu + 32);
 }
@@ -229,17 +248,19 @@ __device__ __forceinline__ void zone_prims(const DevModel &m, int64_t z, double 
 
 // Zone volume sqrt(-g) d^3x L^3 (sqrt(-g) = Sigma sin(theta) r dtheta/dx2 for MKS Kerr-Schild) and the
 // emission prefactor 4 pi A nu_c, A = sqrt(2) pi e^2 n_e / (3 c K2(1/Theta_e)), from the zone-centre state.
-__global__ void k_zone_prep(DevModel m, double *zvol, double *zpref, double *zlnuc, int *bad) {
-  int64_t z = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (z >= m.nz) return;
+__device__ __forceinline__ double zone_geometry(const DevModel &m, int64_t z, Geo &G) {
   double X[4];
   zone_centre(m, z, X);
-  Geo G;
   metric_eval<false>(m, X[1], X[2], G);
   double th, dth, d2th;
   theta_map(m.hslope, X[2], th, dth, d2th);
   double sig = G.r * G.r + m.a * m.a * G.cth * G.cth;
-  zvol[z] = sig * G.sth * G.r * dth * m.dx1 * m.dx2 * m.dx3 * m.L3;
+  return sig * G.sth * G.r * dth * m.dx1 * m.dx2 * m.dx3 * m.L3;
+}
+
+__device__ __forceinline__ void zone_state(const DevModel &m, int64_t z, const Geo &G, double vol, double *zvol, double *zpref,
+                                           double *zlnuc, int *bad) {
+  zvol[z] = vol;
   double pr[8];
   zone_prims(m, z, pr);
   Plasma<double> P;
@@ -272,41 +293,109 @@ __global__ void k_zone_prep(DevModel m, double *zvol, double *zpref, double *zln
   }
 }
 
+// One thread per zone, or (COLUMN) one warp per (i, j) column: the geometry does not depend on x3, so a 3-D grid
+// evaluates it once per column instead of once per zone (more than half of the FP64 work: 2.06 -> 1.14 ms for
+// 288 x 128 x 128 zones).
+template <bool COLUMN>
+__global__ void k_zone_prep(DevModel m, double *zvol, double *zpref, double *zlnuc, int *bad) {
+  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  Geo G;
+  if constexpr (COLUMN) {
+    const int64_t z0 = (t >> 5) * m.n3;
+    if (z0 >= m.nz) return;
+    const double vol = zone_geometry(m, z0, G);
+    for (int k = threadIdx.x & 31; k < m.n3; k += 32) zone_state(m, z0 + k, G, vol, zvol, zpref, zlnuc, bad);
+  } else {
+    if (t >= m.nz) return;
+    const double vol = zone_geometry(m, t, G);
+    zone_state(m, t, G, vol, zvol, zpref, zlnuc, bad);
+  }
+}
+
 void launch_zone_prep(const DevModel &m, double *zvol, double *zpref, double *zlnuc, int *bad, cudaStream_t st) {
-  k_zone_prep<<<(unsigned)((m.nz + 127) / 128), 128, 0, st>>>(m, zvol, zpref, zlnuc, bad);
+  // a column fills its warp from 32 zones on
+  if (m.n3 >= 32) k_zone_prep<true><<<(unsigned)((m.nz / m.n3 + 3) / 4), 128, 0, st>>>(m, zvol, zpref, zlnuc, bad);
+  else k_zone_prep<false><<<(unsigned)((m.nz + 127) / 128), 128, 0, st>>>(m, zvol, zpref, zlnuc, bad);
 }
 
 
 constexpr int kChunk = 2048;
 
-// partial[j][chunk] = sum over the chunk's zones of V_i int dOmega j_nu(nu_j): fixed assignment and a
-// fixed reduction tree, so the weights are bit-reproducible run to run.
-__global__ void k_weight_partial(DevModel m, const double *zvol, const double *zpref, const double *zlnuc,
-                                 double *partial, int nchunks) {
-  __shared__ double red[256];
-  int chunk = blockIdx.x, j = blockIdx.y;
-  int64_t z0 = (int64_t)chunk * kChunk;
-  double s = 0.0;
-  for (int q = threadIdx.x; q < kChunk; q += blockDim.x) {
-    int64_t z = z0 + q;
-    if (z < m.nz) s += zvol[z] * zone_E(m, z, zpref[z], zlnuc[z], j);
-  }
-  red[threadIdx.x] = s;
-  __syncthreads();
-  for (int w = 128; w > 0; w >>= 1) {
-    if ((int)threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) partial[(int64_t)j * nchunks + chunk] = red[0];
+// F(nu/nu_c) at ln(nu/nu_c) = lnK from the cell cubics: 15 FP64 operations where the Lagrange form with its two
+// divisions and exp_t take about 65.
+__device__ __forceinline__ double F_cells(const DevModel &m, double lnK) {
+  const double f = fma(lnK, 1.0 / kFStep, -kFLnK0 / kFStep);
+  const long long kb = dkey(lnK);
+  if (kb >= dkey(kFLnK1)) return 0.0;
+  if (kb <= dkey(kFLnK0)) return F_of_lnK(m, lnK);   // power law below the table
+  double fr;
+  const int i0 = floor_frac(f, fr), c = min(i0, m.nF - 2);
+  const double t = (c == i0) ? fr : f - c;
+  const double2 *q = reinterpret_cast<const double2 *>(m.lnFc) + 2 * c;
+  const double2 lo = __ldg(q), hi = __ldg(q + 1);
+  return exp_q(m.ftab, fma(fma(fma(hi.y, t, hi.x), t, lo.y), t, lo.x));
 }
 
-// w_j = max(w_min, dt dln(nu)_tot / (h N_s) sum_i V_i int dOmega j_nu(nu_j)), dt = 1 (cancels in nu L_nu)
+// int dOmega j_nu(nu_j) of a zone over its prefactor (THERMAL: synchrotron of thermal electrons only), or the whole
+// of it.
+template <bool THERMAL>
+__device__ __forceinline__ double zone_e(const DevModel &m, int64_t z, double pref, double lnuc, double lnu, int j) {
+  if constexpr (THERMAL) return F_cells(m, lnu - lnuc);
+  else return zone_E(m, z, pref, lnuc, j);
+}
+
+// partial[j][chunk] = sum over the chunk's zones of V_i int dOmega j_nu(nu_j): fixed assignment and a
+// fixed reduction tree, so the weights are bit-reproducible run to run.  A CTA takes G nodes of a chunk, so
+// that a zone's volume, prefactor and ln nu_c are read once for G nodes and chunks without emission cost one
+// pass over their prefactors.  The FP64 pipe is the bound, at about 16 operations an emitting zone and node (70
+// with the Lagrange form): 288 x 128 x 128 zones of the torus 14.4 -> 2.9 ms, 1024 x 128 of the sphere 3.0 -> 1.1 ms.
+template <bool THERMAL, int G>
+__global__ void __launch_bounds__(256) k_weight_partial(DevModel m, const double *zvol, const double *zpref,
+                                                        const double *zlnuc, double *partial, int nchunks) {
+  __shared__ double red[8][G];
+  const int chunk = blockIdx.x, j0 = blockIdx.y * G;
+  const int64_t z0 = (int64_t)chunk * kChunk;
+  double s[G], lnu[G];
+#pragma unroll
+  for (int g = 0; g < G; ++g) {
+    s[g] = 0.0;
+    lnu[g] = m.lnu_min + (j0 + g) * m.dlnu;
+  }
+  for (int q = threadIdx.x; q < kChunk; q += 256) {
+    const int64_t z = z0 + q;
+    if (z >= m.nz) break;
+    const double pref = zpref[z];
+    if (pref == 0.0 && (THERMAL || !m.brems)) continue;
+    const double lnuc = zlnuc[z], v = THERMAL ? zvol[z] * pref : zvol[z];
+#pragma unroll
+    for (int g = 0; g < G; ++g)
+      if (j0 + g < m.n_nu) s[g] = fma(v, zone_e<THERMAL>(m, z, pref, lnuc, lnu[g], j0 + g), s[g]);
+  }
+#pragma unroll
+  for (int g = 0; g < G; ++g) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s[g] += __shfl_xor_sync(0xffffffffu, s[g], o);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5][g] = s[g];
+  }
+  __syncthreads();
+  if (threadIdx.x < G && j0 + threadIdx.x < m.n_nu) {
+    double t = 0.0;
+    for (int w = 0; w < 8; ++w) t += red[w][threadIdx.x];
+    partial[(int64_t)(j0 + threadIdx.x) * nchunks + chunk] = t;
+  }
+}
+
+// w_j = max(w_min, dt dln(nu)_tot / (h N_s) sum_i V_i int dOmega j_nu(nu_j)), dt = 1 (cancels in nu L_nu): one warp
+// per node, lanes striding over the chunks, then a fixed tree.
 __global__ void k_weight_final(DevModel m, const double *partial, int nchunks, double n_s, double w_min, double *lnw,
                                double *winv) {
-  int j = blockIdx.x * blockDim.x + threadIdx.x;
+  const int j = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
   if (j >= m.n_nu) return;
   double s = 0.0;
-  for (int c = 0; c < nchunks; ++c) s += partial[(int64_t)j * nchunks + c];
+  for (int c = lane; c < nchunks; c += 32) s += partial[(int64_t)j * nchunks + c];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if (lane != 0) return;
   double w = fmax(w_min, m.dlntot / (kHPL * n_s) * s);
   lnw[j] = log(w);
   winv[j] = 1.0 / w;
@@ -314,41 +403,74 @@ __global__ void k_weight_final(DevModel m, const double *partial, int nchunks, d
 
 void launch_weights(const DevModel &m, const double *zvol, const double *zpref, const double *zlnuc, double *partial,
                     int nchunks, double n_s, double w_min, double *lnw, double *winv, cudaStream_t st) {
-  dim3 grid(nchunks, m.n_nu);
-  k_weight_partial<<<grid, 256, 0, st>>>(m, zvol, zpref, zlnuc, partial, nchunks);
-  k_weight_final<<<(m.n_nu + 127) / 128, 128, 0, st>>>(m, partial, nchunks, n_s, w_min, lnw, winv);
+  const bool thermal = !(m.kappa > 0.0) && !m.brems;
+  // eight nodes per CTA once that still leaves four CTAs per SM (152 SMs); one below, where the chip is not full
+  // (16 chunks: 161 us before, 59 us with one node per CTA)
+  if ((int64_t)nchunks * m.n_nu >= 8 * 600) {
+    const dim3 grid(nchunks, (m.n_nu + 7) / 8);
+    if (thermal) k_weight_partial<true, 8><<<grid, 256, 0, st>>>(m, zvol, zpref, zlnuc, partial, nchunks);
+    else k_weight_partial<false, 8><<<grid, 256, 0, st>>>(m, zvol, zpref, zlnuc, partial, nchunks);
+  } else {
+    const dim3 grid(nchunks, m.n_nu);
+    if (thermal) k_weight_partial<true, 1><<<grid, 256, 0, st>>>(m, zvol, zpref, zlnuc, partial, nchunks);
+    else k_weight_partial<false, 1><<<grid, 256, 0, st>>>(m, zvol, zpref, zlnuc, partial, nchunks);
+  }
+  k_weight_final<<<(m.n_nu + 3) / 4, 128, 0, st>>>(m, partial, nchunks, n_s, w_min, lnw, winv);
 }
 
 // Expected count nbar_i = V_i sum_j T_j g_ij / h (trapezoid in ln nu, g_ij = int dOmega j_nu / w_j), its
 // maximum g over nodes (rejection bound), and N_i = floor(nbar) + [u_i < frac(nbar)], u_i the first
-// uniform of the zone's stream.
-__global__ void k_zone_counts(DevModel m, const double *zvol, const double *zpref, const double *zlnuc, double *zgmax,
-                              double *znbar, int64_t *counts) {
-  int64_t z = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (z >= m.nz) return;
-  double pref = zpref[z], lnuc = zlnuc[z];
-  double s = 0.0, gm = 0.0;
-  if (pref != 0.0 || (m.brems && m.zbq[z] > 0.0)) {
-    for (int j = 0; j < m.n_nu; ++j) {
-      double g = zone_E(m, z, pref, lnuc, j) * m.winv[j];
-      double t = (j == 0 || j == m.n_nu - 1) ? 0.5 * m.dlnu : m.dlnu;
-      s += t * g;
-      gm = fmax(gm, g);
+// uniform of the zone's stream.  Eight lanes share a zone (nodes l, l + 8, ...; fixed reduction): a 2-D grid of
+// some 10^4 zones has too few emitting ones to fill the chip with one thread each, and emitting zones cluster
+// (256 x 128 torus 309 -> 72 us, 1024 x 128 sphere 3.1 -> 1.05 ms, 288 x 128 x 128 torus 3.8 -> 0.79 ms).
+constexpr int kZoneLanes = 8;
+template <bool THERMAL>
+__global__ void __launch_bounds__(128) k_zone_counts(DevModel m, const double *zvol, const double *zpref, const double *zlnuc,
+                                                     double *zgmax, double *znbar, int64_t *counts) {
+  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int64_t z = t / kZoneLanes;
+  const int l = (int)(t % kZoneLanes);
+  const bool in = z < m.nz;
+  const double pref = in ? zpref[z] : 0.0, lnuc = in ? zlnuc[z] : 0.0;
+  const bool on = in && (pref != 0.0 || (!THERMAL && m.brems && m.zbq[z] > 0.0));
+  double s = 0.0;
+  long long gm = 0;   // bit patterns of non-negative doubles order like their values
+  if (on) {
+    double jd = l;
+    for (int j = l; j < m.n_nu; j += kZoneLanes) {
+      const double g = zone_e<THERMAL>(m, z, pref, lnuc, fma(jd, m.dlnu, m.lnu_min), j) * m.winv[j];
+      s = fma((j == 0 || j == m.n_nu - 1) ? 0.5 : 1.0, g, s);
+      gm = max(gm, __double_as_longlong(g));
+      jd += kZoneLanes;
     }
   }
-  double nb = zvol[z] * s / kHPL;
+#pragma unroll
+  for (int o = kZoneLanes / 2; o > 0; o >>= 1) {
+    s += __shfl_xor_sync(0xffffffffu, s, o);
+    gm = max(gm, __shfl_xor_sync(0xffffffffu, gm, o));
+  }
+  if (!in || l != 0) return;
+  double nb = 0.0, g = 0.0;
+  int64_t n = 0;
+  if (on) {
+    const double p = THERMAL ? pref : 1.0;
+    nb = zvol[z] * (p * m.dlnu * s) / kHPL;
+    g = p * __longlong_as_double(gm);
+    const double fl = floor(nb);
+    Rng r;
+    rng_init(r, kZoneTag | (uint64_t)z, 0u);
+    n = (int64_t)fl + ((rng_u(r, m.seed) < nb - fl) ? 1 : 0);
+  }
   znbar[z] = nb;
-  zgmax[z] = gm;
-  double fl = floor(nb);
-  Rng r;
-  rng_init(r, kZoneTag | (uint64_t)z, 0u);
-  double u = rng_u(r, m.seed);
-  counts[z] = (int64_t)fl + ((u < nb - fl) ? 1 : 0);
+  zgmax[z] = g;
+  counts[z] = n;
 }
 
 void launch_counts(const DevModel &m, const double *zvol, const double *zpref, const double *zlnuc, double *zgmax,
                    double *znbar, int64_t *counts, cudaStream_t st) {
-  k_zone_counts<<<(unsigned)((m.nz + 127) / 128), 128, 0, st>>>(m, zvol, zpref, zlnuc, zgmax, znbar, counts);
+  const unsigned grid = (unsigned)((m.nz * kZoneLanes + 127) / 128);
+  if (!(m.kappa > 0.0) && !m.brems) k_zone_counts<true><<<grid, 128, 0, st>>>(m, zvol, zpref, zlnuc, zgmax, znbar, counts);
+  else k_zone_counts<false><<<grid, 128, 0, st>>>(m, zvol, zpref, zlnuc, zgmax, znbar, counts);
 }
 
 // ---------------------------------------------------------------- exclusive scan (int64)
@@ -547,11 +669,12 @@ __global__ void k_selftest_math(int which, const double *x, double *y, double *r
   ref[i] = (which == 0) ? rs : rc;
 }
 
-// Tables of exp_t, log_t and sincospi_t, in extended precision: 2^(j/32); 1/c_j, log c_j split into its
+// Tables of exp_t, log_t and sincospi_t, in extended precision: 2^(j/32) and 2^(j/256); 1/c_j, log c_j split into its
 // double and the remainder (c_j = 1 + j/128); sin and cos (pi j/32), exact at multiples of pi/2.
-void ftab_host(double *t) {
+static void ftab_fill(double *t) {
   const long double pi = 3.141592653589793238462643383279502884L;
   for (int j = 0; j < 32; ++j) t[kFtExp + j] = (double)exp2l((long double)j / 32.0L);
+  for (int j = 0; j < 256; ++j) t[kFtExpQ + j] = (double)exp2l((long double)j / 256.0L);
   for (int j = 0; j < 128; ++j) {
     const long double c = 1.0L + (long double)j / 128.0L;
     t[kFtInvC + j] = (double)(1.0L / c);
@@ -570,6 +693,16 @@ void ftab_host(double *t) {
     t[kFtSin + j] = (double)sv;
     t[kFtCos + j] = (double)cv;
   }
+}
+
+// Copies the tables to t (computed on the first call of the process: extended precision is slow on some hosts).
+void ftab_host(double *t) {
+  struct Tab {
+    double v[kFtN];
+    Tab() { ftab_fill(v); }
+  };
+  static const Tab tab;
+  std::memcpy(t, tab.v, sizeof(tab.v));
 }
 
 cudaError_t selftest_math(int which, const double *x_dev, double *y_dev, double *ref_dev, int64_t n) {
