@@ -163,6 +163,9 @@ DevModel make_model(const mc_ctx *c) {
   m.kapA = c->kapA;
   m.kapI = c->kapI;
   m.kapH = c->kapH;
+  m.gam2 = 2.0 * (p.gam - 1.0);
+  m.cthe = (kMP / kME) * (p.gam - 1.0);
+  m.hCcoef = 0.5 * m.Ccoef;
   m.a2 = p.a * p.a;
   m.twoa = 2.0 * p.a;
   m.M2 = 2.0 * p.mass;
@@ -204,6 +207,8 @@ DevModel make_model(const mc_ctx *c) {
   m.zbnt = c->zbnt;
   m.lnF = c->lnF;
   m.lnFc = c->lnFc;
+  m.lnK2c = c->lnK2c;
+  m.hotc = c->hotc;
   m.nF = c->nF;
   m.lnK2 = c->lnK2;
   m.nK2 = c->nK2;
@@ -296,6 +301,8 @@ int mc_init_model(mc_ctx **out, const mc_model_params *p) {
   c->lnF = (double *)dev_alloc(c, sizeof(double) * c->nF);
   c->lnFc = (double *)dev_alloc(c, sizeof(double) * 4 * (c->nF - 1));
   c->lnK2 = (double *)dev_alloc(c, sizeof(double) * c->nK2);
+  c->lnK2c = (double *)dev_alloc(c, sizeof(double) * 4 * (c->nK2 - 1));
+  c->hotc = (double *)dev_alloc(c, sizeof(double) * 4 * (kHotNT - 1) * (kHotNE - 1));
   c->lnK2f = (float *)dev_alloc(c, sizeof(float) * c->nK2);
   c->hotf = (float *)dev_alloc(c, sizeof(float) * kHotNT * kHotNE);
   c->hot = (double *)dev_alloc(c, sizeof(double) * kHotNT * kHotNE);
@@ -309,7 +316,7 @@ int mc_init_model(mc_ctx **out, const mc_model_params *p) {
   c->lnw = (double *)dev_alloc(c, sizeof(double) * p->n_nu);
   c->winv = (double *)dev_alloc(c, sizeof(double) * p->n_nu);
   c->bad = (int *)dev_alloc(c, sizeof(int));
-  if (!c->lnF || !c->lnFc || !c->lnK2 || !c->hot || !c->gl || !c->cnt || !c->total_dev || !c->spec || !c->lnw || !c->winv || !c->bad) {
+  if (!c->lnF || !c->lnFc || !c->lnK2 || !c->lnK2c || !c->hotc || !c->hot || !c->gl || !c->cnt || !c->total_dev || !c->spec || !c->lnw || !c->winv || !c->bad) {
     mc_free(c);
     return fail(nullptr, MC_ERR_OOM, "device allocation failed");
   }
@@ -358,7 +365,7 @@ int mc_init_model(mc_ctx **out, const mc_model_params *p) {
     launch_kappa_tables(p->kappa, c->kapF, c->kapJ, c->kapA, c->kapI, c->kapH, c->gl + 256, 0);
   }
   DevModel m = make_model(c);
-  launch_tables(m, c->lnF, c->lnFc, c->lnK2, c->hot, c->gl, c->gl + 128, c->gl + 256, 0);
+  launch_tables(m, c->lnF, c->lnFc, c->lnK2, c->lnK2c, c->hot, c->hotc, c->gl, c->gl + 128, c->gl + 256, 0);
   if (!c->lnK2f || !c->hotf) {
     mc_free(c);
     return fail(nullptr, MC_ERR_OOM, "device allocation failed");
@@ -851,7 +858,7 @@ int mc_get_bias_scales(mc_ctx *c, double *scales, int n) {
 }
 
 int mc_selftest_math(int which, const double *x, double *y, double *ref, int64_t n) {
-  if (which < 0 || which > 10 || n < 0 || (n > 0 && (!x || !y || !ref))) return fail(nullptr, MC_ERR_INVALID_ARG, "bad argument");
+  if (which < 0 || which > 18 || n < 0 || (n > 0 && (!x || !y || !ref))) return fail(nullptr, MC_ERR_INVALID_ARG, "bad argument");
   int ndev = 0;
   if (cudaGetDeviceCount(&ndev) != cudaSuccess || ndev < 1) {
     cudaGetLastError();

@@ -82,8 +82,9 @@ __device__ __forceinline__ double dmax_nn(double a, double b) {
 // host in extended precision (ftab_host).  Measured on GB300, in FP64-pipe FMA-equivalents per call:
 // exp 10.9 against 15.1 for CUDA's, log 14.8 against 28.7.  Checked against CUDA's functions by
 // mc_selftest_math.
-constexpr int kFtExp = 0, kFtInvC = 32, kFtLogHi = 160, kFtLogLo = 288, kFtSin = 416, kFtCos = 480, kFtExpQ = 544,
-              kFtN = 800;
+constexpr int kFtExp = 0, kFtInvC = 32, kFtLogHi = 160, kFtLogLo = 288, kFtSin = 416, kFtCos = 480;
+// larger tables of the push and generation kernels' exp_q, log_q (pairs) and sincospi_q (pairs)
+constexpr int kFtExpQ = 544, kFtExpm1Q = 800, kFtLogQ = 1056, kFtSinQ = 3104, kFtN = 7200;
 void ftab_host(double *t);
 
 // e^x = 2^m 2^(j/32) e^r with x = (32 m + j) ln2/32 + r, |r| <= ln2/64 (n = 32 m + j by the 1.5 * 2^52
@@ -124,6 +125,31 @@ __device__ __forceinline__ double exp_q(const double *T, double x) {
   const double tj = __ldg(T + kFtExpQ + (n & 255));
   const double y = fma(tj, pm1, tj);
   return __hiloint2double(__double2hiint(y) + ((n >> 8) << 20), __double2loint(y));
+}
+
+// e^x - 1 for x >= 0 (other arguments: expm1_t): with x = (256 m + j) ln2/256 + r as in exp_q, one r term more for
+// the relative accuracy at small x, and for m = 0 the table holds 2^(j/256) - 1 itself, so nothing cancels:
+// 11 FP64 operations on every branch, where the series and exp_t of expm1_t cost 12 + 12 in a warp that needs
+// both.
+__device__ __forceinline__ double expm1_t(const double *T, double x);
+__device__ __forceinline__ double expm1_q(const double *T, double x) {
+  const long long b = __double_as_longlong(x);
+  if (!(b >= 0 && b < 0x4086200000000000LL)) return expm1_t(T, x);   // 0 <= x < 708
+  const double sh = 6755399441055744.0;
+  const double t = fma(x, 369.3299304675746, sh);
+  const int n = __double2loint(t);
+  const double nd = t - sh;
+  double r = fma(nd, -0.00270760617331689, x);
+  r = fma(nd, -7.453964567463233e-13, r);
+  double q = fma(r, 1.0 / 120.0, 1.0 / 24.0);
+  q = fma(q, r, 1.0 / 6.0);
+  q = fma(q, r, 0.5);
+  const double pm1 = fma(q, r * r, r);
+  const int j = n & 255;
+  const double tj = __ldg(T + kFtExpQ + j);
+  if (n < 256) return fma(tj, pm1, __ldg(T + kFtExpm1Q + j));
+  const double y = fma(tj, pm1, tj);
+  return __hiloint2double(__double2hiint(y) + ((n >> 8) << 20), __double2loint(y)) - 1.0;
 }
 
 // e^x - 1: for |x| < 1/4 its Taylor series to x^12 (truncation below 1e-17 relative), by Horner in
@@ -171,6 +197,40 @@ __device__ __forceinline__ double log_t(const double *T, double x) {
   const double ed = __hiloint2double(0x43300000, (int)(0x80000000u + (unsigned)e)) - 4503601774854144.0;   // (double)e
   const double kLn2Hi = 0.69314718055920821, kLn2Lo = 7.3710025651677989e-13;   // ln2: 40 significant bits + rest
   return fma(ed, kLn2Hi, __ldg(T + kFtLogHi + j)) + (l1p + fma(ed, kLn2Lo, __ldg(T + kFtLogLo + j)));
+}
+
+// log x with c = 1 + (j + 1/2)/1024 from the top 10 mantissa bits: |r| < 1/2048, series to r^4 (truncation below
+// 6e-18), ln2 and log c as single doubles: 9 FP64 operations instead of 15, absolute error within ~1 ulp of the
+// largest term (the callers interpolate tables in it).
+__device__ __forceinline__ double log_q(const double *T, double x) {
+  const long long b = __double_as_longlong(x);
+  if (!(b >= 0x0010000000000000LL && b < 0x7FF0000000000000LL)) return log(x);
+  const int hi = (int)(b >> 32);
+  const int e = (hi >> 20) - 1023;
+  const int j = (hi >> 10) & 1023;
+  const double m = __hiloint2double((hi & 0x000fffff) | 0x3ff00000, (int)b);
+  const double c = __hiloint2double(0x3ff00000 | (j << 10) | (1 << 9), 0);
+  const double2 tc = __ldg(reinterpret_cast<const double2 *>(T + kFtLogQ) + j);   // 1 / c, log c
+  const double r = (m - c) * tc.x;
+  const double q = fma(fma(r, -0.25, 1.0 / 3.0), r, -0.5);
+  const double l1p = fma(q, r * r, r);
+  const double ed = __hiloint2double(0x43300000, (int)(0x80000000u + (unsigned)e)) - 4503601774854144.0;   // (double)e
+  return fma(ed, 0.693147180559945309, tc.y) + l1p;
+}
+
+// sin(pi x), cos(pi x) from a table of pi j/1024 (|pi r| <= pi/2048: two-term series, truncation below 2e-20): 14
+// FP64 operations instead of 18.  The part of the table in use (x in [0, 1/2] in the point geometry) is 8 KB.
+__device__ __forceinline__ void sincospi_q(const double *T, double x, double &s, double &c) {
+  const double sh = 6755399441055744.0;
+  const double t = fma(x, 1024.0, sh);
+  const int j = __double2loint(t) & 2047;
+  const double r = fma(t - sh, -0.0009765625, x);
+  const double a = __dmul_rn(r, 3.141592653589793), a2 = __dmul_rn(a, a);
+  const double sa = fma(__dmul_rn(a, a2), fma(a2, 1.0 / 120.0, -1.0 / 6.0), a);
+  const double ca = fma(a2, fma(a2, 1.0 / 24.0, -0.5), 1.0);
+  const double2 tj = __ldg(reinterpret_cast<const double2 *>(T + kFtSinQ) + j);   // sin, cos
+  s = fma(tj.x, ca, __dmul_rn(tj.y, sa));
+  c = fma(tj.y, ca, -__dmul_rn(tj.x, sa));
 }
 
 // sin(pi x), cos(pi x): x = n/32 + r exactly (|r| <= 1/64, n by the 1.5 * 2^52 shift), the angle-addition
@@ -268,7 +328,7 @@ struct DevModel {
   const float *prim32x;   // FP32 primitives for the FP32 coefficient path (the grid or a copy), or NULL
   // tables
   const double *lnF;      // angle integral
-  const double *lnFc;     // its cubics per cell (see F_cells)
+  const double *lnFc, *lnK2c, *hotc;   // cell polynomials: cubics of lnF and lnK2, bilinear forms of hot
   int nF;
   const double *lnK2;
   int nK2;
@@ -279,6 +339,7 @@ struct DevModel {
   int brems;              // thermal bremsstrahlung on
   df dmass, da, dx1_0, dx1_hi, dr_record, dr_capture;   // double-float splits for the mixed geodesic
   df dpi2hh, dhh_pi, dd2th;   // pi (1 - h), (1 - h) / (2 pi), -2 pi^2 (1 - h): the theta map in double-float
+  double gam2, cthe, hCcoef;   // 2 (gam - 1), (m_p / m_e) (gam - 1), Ccoef / 2
   double a2, twoa, M2, pi2hh, hh_pi2, d2th2;   // a^2, 2 a, 2 M and the theta map's pi (1-h), (1-h) / pi, -4 pi^2 (1-h)
   const df *dtab;             // double-float function table (kDfTabN entries)
   float fidx1, fidx2, fidx3, fx2_0, fx3_0;   // FP32 grid constants for the double-float zone lookup
@@ -692,9 +753,9 @@ template <bool KERR = true>
 __device__ __forceinline__ void point_eval(const DevModel &m, double x1, double x2, Point &G) {
   const bool far = upper_half(x2);
   const double y = far ? ssub(1.0, x2) : x2;
-  G.r = exp_t(m.ftab, x1);
+  G.r = exp_q(m.ftab, x1);
   double sp, cp;
-  sincospi_t(m.ftab, y, sp, cp);
+  sincospi_q(m.ftab, y, sp, cp);
   if (m.hslope1) {
     G.s = sp;
     G.c = cp;
@@ -705,7 +766,7 @@ __device__ __forceinline__ void point_eval(const DevModel &m, double x1, double 
     const double sc1 = smul(sp, cp);                                         // sin(2 pi y) / 2
     G.dth = mad(m.pi2hh, smul(ssub(cp, sp), sadd(cp, sp)), kPI);   // pi (1 + (1-h) cos(2 pi y))
     G.d2th = smul(m.d2th2, sc1);                     // -2 pi^2 (1-h) sin(2 pi y)
-    sincospi_t(m.ftab, mad(m.hh_pi2, sc1, y), G.s, G.c);
+    sincospi_q(m.ftab, mad(m.hh_pi2, sc1, y), G.s, G.c);
     G.idth = rcp_n(G.dth);
   }
   if (far) {
@@ -956,6 +1017,49 @@ __device__ __forceinline__ double pow_sixth(double X) {
   }
   const double z2 = z * z;
   return X * (z2 * z2 * z);
+}
+
+// The same by one step: with the seed z ~ X^(-1/6) (narrowed and widened on the integer pipes), s = X z^5 and
+// t = 1 - s z = 1 - X z^6 (about 6 times the seed's relative error, < 1e-5), X^(1/6) = s (1 - t)^(-5/6) to t^3:
+// 9 FP64 operations instead of 18 with two conversions.
+__device__ __forceinline__ double sixth_root(double X) {
+  if (!(__double_as_longlong(X) > 0x39B4484BFEEBC2A0LL && __double_as_longlong(X) < 0x46293E5939A08CEALL)) return pow_sixth(X);
+  const double z = widen_exact(__expf(__logf(narrow_f(X)) * (-1.0f / 6.0f)));
+  const double z2 = z * z, s = X * (z2 * z2 * z);
+  const double t = fma(-s, z, 1.0);
+  double q = fma(t, 935.0 / 1296.0, 55.0 / 72.0);
+  q = fma(q, t, 5.0 / 6.0);
+  return fma(s * t, q, s);
+}
+
+// Cubic of a cell table (see k_cubic_cells) at index coordinate f, extended past its ends like cubic_table.
+__device__ __forceinline__ double cell_cubic(const double *cells, int ncell, double f) {
+  double fr;
+  const int i0 = floor_frac(f, fr), c = max(0, min(i0, ncell - 1));
+  const double t = (c == i0) ? fr : f - c;
+  const double2 *q = reinterpret_cast<const double2 *>(cells) + 2 * c;
+  const double2 lo = __ldg(q), hi = __ldg(q + 1);
+  return fma(fma(fma(hi.y, t, hi.x), t, lo.y), t, lo.x);
+}
+
+__device__ __forceinline__ double lnK2_cells(const DevModel &m, double lt) {
+  if (m.k2_mode == 1) return fma(2.0, lt, 0.6931471805599453);   // ln(2 Theta^2)
+  return cell_cubic(m.lnK2c, m.nK2 - 1, fma(lt, 1.0 / kK2Step, -kK2LnT0 / kK2Step));
+}
+
+// sigma_h / sigma_T: bilinear in (ln Theta, ln eps) as hot_lookup_ln, from v00, dv/db, dv/da, d2v/dadb of the cell.
+__device__ __forceinline__ double hot_cells(const DevModel &m, double lt, double le) {
+  constexpr double st = (kHotNT - 1) / (kHotLT1 - kHotLT0), se = (kHotNE - 1) / (kHotLE1 - kHotLE0);
+  const double ft = dmin_nn(dmax0(fma(lt, st, -kHotLT0 * st)), (double)(kHotNT - 1));
+  const double fe = dmin_nn(dmax0(fma(le, se, -kHotLE0 * se)), (double)(kHotNE - 1));
+  double a, b;
+  const int i0 = floor_frac(ft, a), j0 = floor_frac(fe, b);
+  const int i = min(i0, kHotNT - 2), j = min(j0, kHotNE - 2);
+  if (i != i0) a = 1.0;   // at the last node
+  if (j != j0) b = 1.0;
+  const double2 *q = reinterpret_cast<const double2 *>(m.hotc) + 2 * (i * (kHotNE - 1) + j);
+  const double2 lo = __ldg(q), hi = __ldg(q + 1);
+  return exp_q(m.ftab, fma(a, fma(b, hi.y, hi.x), fma(b, lo.y, lo.x)));
 }
 
 // ---------------------------------------------------------------- kappa electrons (future work in section 6)
@@ -1325,57 +1429,110 @@ struct CoefT {
 };
 using Coef = CoefT<double>;
 
-__device__ __forceinline__ void coefficients64(const DevModel &m, const Geo &G, const double X[4], const double K[4],
+// FP64 form, from the point geometry.  The spatial metric of g = g0 + f l l is diagonal in the covectors l,
+// d theta and d phi: V.W = (1 + f) (lV)(lW) + Sigma (V^th W^th + sin^2 V^ph W^ph) with lV = V^r - a sin^2 V^ph, so
+// the products below need no metric component and no lowered 4-vector.  With U the velocity and B the field
+// relative to the normal observers (lapse (1 + f)^-1/2):
+//   gamma^2 = 1 + U.U, u^t = gamma (1 + f)^1/2, b^t = B.U, b^2 = (B.B + (B.U)^2) / (u^t)^2,
+//   eps = -k.u = gamma (1 + f)^-1/2 k^t - k_i U^i, k.b = (k_i B^i - (B.U) eps) / u^t,
+//   k_i V^i = (l_i k^i + f L) lV + Sigma (k^th V^th + sin^2 k^ph V^ph).
+// About 200 FP64 operations with the interpolation, log and exp calls, where lowering u, b and k and the
+// table forms took about 340; reciprocals and roots take one third-order step each (rcp_n, rsqrt_n).  The FP64
+// pipe is the bound: with the shorter sincospi and exp of the point geometry the in-grid phase of a 3-D snapshot
+// shard went from 330 to 275 ms and the 2-D torus's from 256 to 214 ms.
+template <bool KERR>
+__device__ __forceinline__ void coefficients64(const DevModel &m, const Point &G, const double X[4], const double K[4],
                                                bool want_s, Coef &c) {
   c.ana = c.ans = c.thetae = 0.0;
   double pr[8];
   if (!interp_prims<double>(m, X, pr)) return;
-  Plasma<double> P;
-  plasma_from_prims<double>(m, G, pr, P, nullptr, nullptr);
-  c.thetae = P.thetae;
-  if (!P.on) return;
-  double eps = -(K[0] * P.ucov[0] + K[1] * P.ucov[1] + K[2] * P.ucov[2] + K[3] * P.ucov[3]);
-  {
-    const long long be = __double_as_longlong(eps);
-    if (!(be > 0 && be < 0x7FF0000000000000LL)) return;   // eps > 0 (and finite) on the bit pattern
+  const double rho = pr[0], uu = pr[1];
+  const auto pos = [](double x) { return __double_as_longlong(x) > 0 && __double_as_longlong(x) < 0x7FF0000000000000LL; };
+  const bool rho_pos = pos(rho);
+  double lU = G.r * pr[5], lB = G.r * pr[2], lk = G.r * K[1];
+  if constexpr (KERR) {
+    lU = fma(-G.as2, pr[7], lU);
+    lB = fma(-G.as2, pr[4], lB);
+    lk = fma(-G.as2, K[3], lk);
   }
+  const double hU = G.dth * pr[6], hB = G.dth * pr[3], hk = G.dth * K[2];
+  const double opf = 1.0 + G.f, ss2 = G.sig * G.s2;
+  const double pU = opf * lU, tU = G.sig * hU, fU = ss2 * pr[7];
+  const double pB = opf * lB, tB = G.sig * hB, fB = ss2 * pr[4];
+  const double UU = fma(pU, lU, fma(tU, hU, fU * pr[7]));
+  const double BU = fma(pU, lB, fma(tU, hB, fU * pr[4]));
+  const double BB = fma(pB, lB, fma(tB, hB, fB * pr[4]));
+  const double ek = fma(G.f, K[0] + lk, lk);
+  const double kU = fma(ek, lU, fma(hk, tU, K[3] * fU));
+  const double kB = fma(ek, lB, fma(hk, tB, K[3] * fB));
+  const double g2 = 1.0 + UU;
+  const double iut = rsqrt_n(g2 * opf);            // 1 / u^t
+  const double eps = fma(g2 * iut, K[0], -kU);
+  const double bb = fma(BU, BU, BB);               // (u^t)^2 b^2
+  const bool b_pos = pos(bb);
+  const double ib = b_pos ? (bb > 1e-290 ? rsqrt_n(bb) : rsqrt(bb)) : 0.0;
+  const double b2 = b_pos ? bb * (iut * iut) : 0.0;
+  // Theta_e = (m_p/m_e)(gam-1)(u/rho)/(1 + T_i/T_e), T_i/T_e = (R_high beta^2 + R_low)/(1 + beta^2), beta = P / b^2
+  double th = 0.0, ith = 0.0;
+  if (rho_pos && pos(uu)) {
+    const double P = m.gam2 * uu, P2 = P * P, b4 = b2 * b2;
+    const double num = (m.cthe * uu) * (b4 + P2);
+    const double den = rho * fma(1.0 + m.R_high, P2, (1.0 + m.R_low) * b4);
+    const long long nd = __double_as_longlong(num * den);
+    if (nd > __double_as_longlong(1e-280) && nd < __double_as_longlong(1e280)) {
+      // Theta_e and 1/Theta_e from one reciprocal
+      const double inv = rcp_n(__longlong_as_double(nd));
+      th = num * (num * inv);
+      ith = den * (den * inv);
+    } else {   // beta^2 leaves the range: the ratio itself
+      const double beta = b_pos ? P / b2 : 1e150, x = beta * beta;
+      const double r = b_pos && x < 1e300 ? (1.0 + x) / (1.0 + m.R_low + (1.0 + m.R_high) * x) : 1.0 / (1.0 + m.R_high);
+      th = m.cthe * (uu / rho) * r;
+      ith = 1.0 / th;
+    }
+    if (__double_as_longlong(th) > __double_as_longlong(m.thetae_max)) {   // th >= 0
+      th = m.thetae_max;
+      ith = m.ithetae_max;
+    }
+  }
+  c.thetae = th;
+  if (!rho_pos) return;
+  const double ne = rho * m.Ne_unit;
+  if (!pos(eps)) return;
   constexpr double kNuEps = kME * kCL * kCL / kHPL;   // nu / eps
-  const double ieps = 1.0 / eps;
-  double nu = eps * kNuEps;
-  double lt = log_t(m.ftab, dmax_nn(P.thetae, 1e-300));
-  // Theta_e >= Theta_min and a field (B > 0 implies b^2 > 0), as sign / order tests on bit patterns
-  const bool emits = dge_nn(P.thetae, m.thetae_min) && __double_as_longlong(P.B) > 0;
-  if (m.kappa_on && emits) {
-    double kb = K[0] * P.bcov[0] + K[1] * P.bcov[1] + K[2] * P.bcov[2] + K[3] * P.bcov[3];
-    double cth = fmin(1.0, fmax(-1.0, kb * P.rb * ieps));
-    double s2 = 1.0 - cth * cth;
-    if (s2 > 0.0) c.ana = kappa_nu_alpha(m, P.ne, P.thetae, P.B, s2 * rsqrt(s2), nu);
-  } else if (emits) {
-    double kb = K[0] * P.bcov[0] + K[1] * P.bcov[1] + K[2] * P.bcov[2] + K[3] * P.bcov[3];
-    double cth = fmin(1.0, fmax(-1.0, kb * P.rb * ieps));
-    double s2 = 1.0 - cth * cth;
-    if (__double_as_longlong(s2) > 0) {   // s2 > 0 (s2 <= 1)
-      constexpr double kNus = (2.0 / 9.0) * (kEE / (2.0 * kPI * kME * kCL));   // nu_s / (B Theta^2 sin)
-      const double rs = rsqrt(s2);
-      double nus = kNus * P.B * P.thetae * P.thetae * (s2 * rs);
-      // X = nu / nu_s from the reciprocals at hand: 1/B = rb / B_unit, 1/Theta, 1/sin = rs
-      double Xs = nu * (1.0 / kNus) * (P.rb * m.iB_unit) * (P.ith * P.ith) * rs;
-      // G(X) / K2 with one exponential: G = t^2 exp(-X^1/3), t = X^1/2 + 2^(11/12) X^1/6
-      double x6 = pow_sixth(Xs);
-      double x3 = x6 * x6;
-      if (!dge_nn(x3, 745.0)) {   // x3 < 745; beyond, exp(-X^1/3) underflows: no emission or absorption
-        double t = x6 * x3 + 1.8877486253633870 * x6;
-        double GoK = t * t * exp_t(m.ftab, -x3 - lnK2_of_ln(m, lt));
-        // nu alpha_nu = nu j_nu / B_nu with j_nu = sqrt2 pi e^2 n_e nu_s G / (3 c K2) and
-        // B_nu = 2 h nu^3 / (c^2 expm1(h nu / k T)), h nu / k T = eps / Theta_e:
-        // nu alpha_nu = (sqrt2 pi e^2 c / 6h) n_e (G / K2) expm1(eps/Theta) nu_s / nu^2
-        const double C1 = 1.4142135623730951 * kPI * kEE * kEE * kCL / (6.0 * kHPL) / (kNuEps * kNuEps);
-        c.ana = C1 * P.ne * GoK * expm1_t(m.ftab, eps * P.ith) * nus * (ieps * ieps);
+  const double ieps = rcp_n(eps);
+  const double nu = eps * kNuEps;
+  const double lt = log_q(m.ftab, dmax_nn(th, 1e-300));
+  // Theta_e >= Theta_min and a field
+  if (dge_nn(th, m.thetae_min) && b_pos) {
+    const double B = (bb * ib) * (iut * m.B_unit);
+    const double cth = (fma(-BU, eps, kB) * ib) * ieps;
+    const double s2 = fma(-cth, cth, 1.0);
+    if (__double_as_longlong(s2) > 0) {   // |cos| < 1
+      const double rs = rsqrt_n(s2);
+      if (m.kappa_on) {
+        c.ana = kappa_nu_alpha(m, ne, th, B, s2 * rs, nu);
+      } else {
+        constexpr double kNus = (2.0 / 9.0) * (kEE / (2.0 * kPI * kME * kCL));   // nu_s / (B Theta^2 sin)
+        const double nus = (kNus * B) * (th * th) * (s2 * rs);
+        const double Xs = nu * rcp_n(nus);
+        // G(X) / K2 with one exponential: G = t^2 exp(-X^1/3), t = X^1/2 + 2^(11/12) X^1/6
+        const double x6 = sixth_root(Xs), x3 = x6 * x6;
+        if (!dge_nn(x3, 745.0)) {   // beyond, exp(-X^1/3) underflows: no emission or absorption
+          const double t = fma(x6, x3, 1.8877486253633870 * x6);
+          const double GoK = (t * t) * exp_q(m.ftab, -x3 - lnK2_cells(m, lt));
+          // nu alpha_nu = nu j_nu / B_nu with j_nu = sqrt2 pi e^2 n_e nu_s G / (3 c K2) and
+          // B_nu = 2 h nu^3 / (c^2 expm1(h nu / k T)), h nu / k T = eps / Theta_e:
+          // nu alpha_nu = (sqrt2 pi e^2 c / 6h) n_e (G / K2) expm1(eps/Theta) nu_s / nu^2
+          constexpr double C1 = 1.4142135623730951 * kPI * kEE * kEE * kCL / (6.0 * kHPL) / (kNuEps * kNuEps);
+          c.ana = ((C1 * ne) * GoK) * (expm1_q(m.ftab, eps * ith) * nus) * (ieps * ieps);
+        }
       }
     }
   }
-  if (m.brems) c.ana += brems_nu_alpha(P.ne, P.thetae, nu);
-  if (want_s) c.ans = nu * P.ne * (m.kappa > 0.0 ? kap_hot_lookup(m, P.thetae, eps) : hot_lookup_ln(m, lt, log_t(m.ftab, eps)));
+  if (m.brems) c.ana += brems_nu_alpha(ne, th, nu);
+  if (want_s)
+    c.ans = (nu * ne) * (m.kappa_on ? kap_hot_lookup(m, th, eps) : kSIGT * hot_cells(m, lt, log_q(m.ftab, eps)));
 }
 
 // Mixed precision: the same quantities with FP32 plasma state and coefficient arithmetic.

@@ -76,7 +76,7 @@ struct PushIO {
 };
 
 // tables (mc_tables.cu)
-void launch_tables(const DevModel &m, double *lnF, double *lnFc, double *lnK2, double *hot, const double *gl_ang,
+void launch_tables(const DevModel &m, double *lnF, double *lnFc, double *lnK2, double *lnK2c, double *hot, double *hotc, const double *gl_ang,
                    const double *gl_s, const double *gl_mu, cudaStream_t st);
 // generation (mc_tables.cu)
 void launch_zone_prep(const DevModel &m, double *zvol, double *zpref, double *zlnuc, int *bad, cudaStream_t st);
@@ -116,7 +116,7 @@ struct mc_ctx {
   // allocations made through the caller's allocator (or cudaMalloc)
   std::vector<void *> allocs;
   // tables
-  double *lnF = nullptr, *lnFc = nullptr, *lnK2 = nullptr, *hot = nullptr, *gl = nullptr;
+  double *lnF = nullptr, *lnFc = nullptr, *lnK2 = nullptr, *lnK2c = nullptr, *hotc = nullptr, *hot = nullptr, *gl = nullptr;
   int nF = 0, nK2 = 0;
   // grid
   bool have_grid = false;

@@ -55,12 +55,6 @@ struct LocalStats {
   unsigned long long emit, child, rec, abs, capt, maxst, steps, iters, nonconv, roul, rejcap, events, gsteps, giters;
 };
 
-template <bool C32, typename S, typename W>
-__device__ __forceinline__ void coefs(const DevModel &m, const GeoT<S> &G, const S X[4], const S K[4], bool ws,
-                                      CoefT<W> &c) {
-  if constexpr (C32) coefficients32(m, G, X, K, ws, c);
-  else coefficients64(m, G, X, K, ws, c);
-}
 
 // Geometry of a geodesic step: POINT, the point's Kerr-Schild factors (FP64); otherwise the metric's components
 // and derivatives, in double-float or, in the split form's in-grid steps where a = 0 can occur (single models
@@ -104,13 +98,22 @@ static __device__ void init_transport(const DevModel &m, Ph &p) {
   p.x1t = -log(rng_u(p.s, m.seed));
   p.acc = 0.0;
   bool scat = m.scatter && p.nsc < m.n_sc_max;
-  Geo G;
-  metric_eval<true, KERR>(m, p.X[1], p.X[2], G);
   Coef c;
-  coefs<C32>(m, G, p.X, p.K, scat, c);
-  p.ana = c.ana;
-  p.ans = c.ans;
-  accel<KERR>(G, p.K, p.A);
+  if constexpr (C32) {
+    Geo G;
+    metric_eval<true, KERR>(m, p.X[1], p.X[2], G);
+    coefficients32(m, G, p.X, p.K, scat, c);
+    p.ana = c.ana;
+    p.ans = c.ans;
+    accel<KERR>(G, p.K, p.A);
+  } else {
+    Point G;
+    point_eval<KERR>(m, p.X[1], p.X[2], G);
+    coefficients64<KERR>(m, G, p.X, p.K, scat, c);
+    p.ana = c.ana;
+    p.ans = c.ans;
+    accel<KERR>(m, G, p.K, p.A);
+  }
   p.nsteps = 0;
   p.nev = 0;
   p.wb = p.w;
@@ -692,12 +695,12 @@ __device__ __forceinline__ void absorb_scatter(const DevModel &m, const PushIO &
     }
     p.w = wn;
   } else {
-    const double C = m.Ccoef, dld = to_d(dls);
-    double tau_a = 0.5 * (p.ana + c.ana) * C * dld;
+    const double hC = m.hCcoef * to_d(dls);   // C dl / 2
+    double tau_a = (p.ana + c.ana) * hC;
     double w0 = p.w;
-    double wn = w0 * exp_t(m.ftab, -tau_a);
+    double wn = w0 * exp_q(m.ftab, -tau_a);
     if (scat) {
-      double tau_s = 0.5 * (p.ans + c.ans) * C * dld;
+      double tau_s = (p.ans + c.ans) * hC;
       if (__double_as_longlong(tau_s) > 0) {   // tau_s > 0 (tau_s >= 0)
         double b = bias_of(m, c.thetae, p.nsc);
         double d = b * tau_s;
@@ -818,7 +821,8 @@ static __device__ bool step(const DevModel &m, const PushIO &io, PhF<PREC> &p, L
   p.nsteps++;
   ls.steps++;
   CoefT<W> c;
-  coefs<Form<PREC>::C32>(m, geo_of<KERR>(m, G), p.X, p.K, scat, c);
+  if constexpr (Form<PREC>::C32) coefficients32(m, geo_of<KERR>(m, G), p.X, p.K, scat, c);
+  else coefficients64<KERR>(m, G, p.X, p.K, scat, c);
   absorb_scatter(m, io, p, X0, K0, dl, c, scat, ls);
   const int rt = at_record(m, G.r) ? 1 : (at_capture(m, G.r) ? 3 : 0);
   return terminate<KERR>(m, io, G, p, rt, ls) == 0;

@@ -83,12 +83,26 @@ __global__ void k_cubic_cells(const double *y, int n, double *cell) {
   cell[4 * c + 3] = a3;
 }
 
-void launch_tables(const DevModel &m, double *lnF, double *lnFc, double *lnK2, double *hot, const double *gl_ang, const double *gl_s,
+// Bilinear forms of the hot cross-section table per cell: v00, v01 - v00, v10 - v00, v11 - v10 - v01 + v00.
+__global__ void k_hot_cells(const double *hot, double *cell) {
+  const int c = blockIdx.x * blockDim.x + threadIdx.x;
+  if (c >= (kHotNT - 1) * (kHotNE - 1)) return;
+  const double *h = hot + (c / (kHotNE - 1)) * kHotNE + c % (kHotNE - 1);
+  const double v00 = h[0], v01 = h[1], v10 = h[kHotNE], v11 = h[kHotNE + 1];
+  cell[4 * c] = v00;
+  cell[4 * c + 1] = v01 - v00;
+  cell[4 * c + 2] = v10 - v00;
+  cell[4 * c + 3] = (v11 - v10) - (v01 - v00);
+}
+
+void launch_tables(const DevModel &m, double *lnF, double *lnFc, double *lnK2, double *lnK2c, double *hot, double *hotc, const double *gl_ang, const double *gl_s,
                    const double *gl_mu, cudaStream_t st) {
   k_table_F<<<(m.nF + 127) / 128, 128, 0, st>>>(lnF, m.nF, gl_ang, gl_ang + 64);
   k_cubic_cells<<<(m.nF + 126) / 128, 128, 0, st>>>(lnF, m.nF, lnFc);
   k_table_K2<<<(m.nK2 + 127) / 128, 128, 0, st>>>(lnK2, m.nK2);
+  k_cubic_cells<<<(m.nK2 + 126) / 128, 128, 0, st>>>(lnK2, m.nK2, lnK2c);
   k_table_hot<<<(kHotNT * kHotNE + 127) / 128, 128, 0, st>>>(hot, gl_s, gl_s + 64, gl_mu, gl_mu + 32);
+  k_hot_cells<<<((kHotNT - 1) * (kHotNE - 1) + 127) / 128, 128, 0, st>>>(hot, hotc);
 }
 
 // ---------------------------------------------------------------- kappa electrons
@@ -328,12 +342,7 @@ __device__ __forceinline__ double F_cells(const DevModel &m, double lnK) {
   const long long kb = dkey(lnK);
   if (kb >= dkey(kFLnK1)) return 0.0;
   if (kb <= dkey(kFLnK0)) return F_of_lnK(m, lnK);   // power law below the table
-  double fr;
-  const int i0 = floor_frac(f, fr), c = min(i0, m.nF - 2);
-  const double t = (c == i0) ? fr : f - c;
-  const double2 *q = reinterpret_cast<const double2 *>(m.lnFc) + 2 * c;
-  const double2 lo = __ldg(q), hi = __ldg(q + 1);
-  return exp_q(m.ftab, fma(fma(fma(hi.y, t, hi.x), t, lo.y), t, lo.x));
+  return exp_q(m.ftab, cell_cubic(m.lnFc, m.nF - 1, f));
 }
 
 // int dOmega j_nu(nu_j) of a zone over its prefactor (THERMAL: synchrotron of thermal electrons only), or the whole
@@ -633,6 +642,45 @@ __global__ void k_selftest_math(int which, const double *x, double *y, double *r
     ref[i] = expm1(v);
     return;
   }
+  // the larger-table and one-step forms of the push and generation kernels
+  if (which == 11) {
+    y[i] = exp_q(F, v);
+    ref[i] = exp(v);
+    return;
+  }
+  if (which == 12) {
+    y[i] = log_q(F, v);
+    ref[i] = log(v);
+    return;
+  }
+  if (which == 13 || which == 14) {
+    double s, c, rs, rc;
+    sincospi_q(F, v, s, c);
+    sincospi(v, &rs, &rc);
+    y[i] = which == 13 ? s : c;
+    ref[i] = which == 13 ? rs : rc;
+    return;
+  }
+  if (which == 15) {
+    y[i] = expm1_q(F, v);
+    ref[i] = expm1(v);
+    return;
+  }
+  if (which == 16) {
+    y[i] = sixth_root(v);
+    ref[i] = cbrt(sqrt(v));
+    return;
+  }
+  if (which == 17) {
+    y[i] = rcp_n(v);
+    ref[i] = 1.0 / v;
+    return;
+  }
+  if (which == 18) {
+    y[i] = rsqrt_n(v);
+    ref[i] = rsqrt(v);
+    return;
+  }
   if (which == 8 || which == 9) {
     double s, c, rs, rc;
     sincospi_t(F, v, s, c);
@@ -669,12 +717,30 @@ __global__ void k_selftest_math(int which, const double *x, double *y, double *r
   ref[i] = (which == 0) ? rs : rc;
 }
 
-// Tables of exp_t, log_t and sincospi_t, in extended precision: 2^(j/32) and 2^(j/256); 1/c_j, log c_j split into its
+// Tables of the exp, log and sincospi functions, in extended precision: 2^(j/32), 2^(j/256) and 2^(j/256) - 1; 1/c_j, log c_j split into its
 // double and the remainder (c_j = 1 + j/128); sin and cos (pi j/32), exact at multiples of pi/2.
 static void ftab_fill(double *t) {
   const long double pi = 3.141592653589793238462643383279502884L;
   for (int j = 0; j < 32; ++j) t[kFtExp + j] = (double)exp2l((long double)j / 32.0L);
-  for (int j = 0; j < 256; ++j) t[kFtExpQ + j] = (double)exp2l((long double)j / 256.0L);
+  for (int j = 0; j < 256; ++j) {
+    t[kFtExpQ + j] = (double)exp2l((long double)j / 256.0L);
+    t[kFtExpm1Q + j] = (double)expm1l((long double)j / 256.0L * 0.693147180559945309417232121458176568L);
+  }
+  for (int j = 0; j < 1024; ++j) {
+    const long double c = 1.0L + ((long double)j + 0.5L) / 1024.0L;
+    t[kFtLogQ + 2 * j] = (double)(1.0L / c);
+    t[kFtLogQ + 2 * j + 1] = (double)logl(c);
+  }
+  // sin(pi j/1024) for one octant pair, then by symmetry: exact at multiples of pi/2
+  long double q[513];
+  for (int j = 0; j <= 512; ++j) q[j] = j == 512 ? 1.0L : sinl(pi * j / 1024.0L);
+  for (int j = 0; j < 2048; ++j) {
+    const int u = j % 1024;
+    const long double sv = u <= 512 ? q[u] : q[1024 - u];
+    const long double cv = u <= 512 ? q[512 - u] : -q[u - 512];
+    t[kFtSinQ + 2 * j] = (double)(j < 1024 ? sv : -sv);
+    t[kFtSinQ + 2 * j + 1] = (double)(j < 1024 ? cv : -cv);
+  }
   for (int j = 0; j < 128; ++j) {
     const long double c = 1.0L + (long double)j / 128.0L;
     t[kFtInvC + j] = (double)(1.0L / c);
