@@ -948,16 +948,6 @@ __device__ __forceinline__ double K2_of(const DevModel &m, double thetae) {
   return exp(cubic_table(m.lnK2, m.nK2, kK2LnT0, 1.0 / kK2Step, log(thetae)));
 }
 
-__device__ __forceinline__ double K2_of_ln(const DevModel &m, double thetae, double lt) {
-  if (m.k2_mode == 1) return 2.0 * thetae * thetae;
-  return exp(cubic_table(m.lnK2, m.nK2, kK2LnT0, 1.0 / kK2Step, lt));
-}
-
-__device__ __forceinline__ double lnK2_of_ln(const DevModel &m, double lt) {
-  if (m.k2_mode == 1) return 0.6931471805599453 + 2.0 * lt;   // ln(2 Theta^2)
-  return cubic_table(m.lnK2, m.nK2, kK2LnT0, 1.0 / kK2Step, lt);
-}
-
 __device__ __forceinline__ float K2_of_f(const DevModel &m, float thetae) {
   if (m.k2_mode == 1) return 2.0f * thetae * thetae;
   float f = (__logf(thetae) - (float)kK2LnT0) * (float)(1.0 / kK2Step);
@@ -965,28 +955,6 @@ __device__ __forceinline__ float K2_of_f(const DevModel &m, float thetae) {
   float u = f - i;
   float l = (1.0f - u) * m.lnK2f[i] + u * m.lnK2f[i + 1];
   return __expf(l);
-}
-
-__device__ __forceinline__ double hot_lookup_ln(const DevModel &m, double lt, double le) {
-  constexpr double st = (kHotNT - 1) / (kHotLT1 - kHotLT0), se = (kHotNE - 1) / (kHotLE1 - kHotLE0);
-  double ft = (lt - kHotLT0) * st;
-  double fe = (le - kHotLE0) * se;
-  ft = dmin_nn(dmax0(ft), (double)(kHotNT - 1));
-  fe = dmin_nn(dmax0(fe), (double)(kHotNE - 1));
-  double a, b;
-  const int i0 = floor_frac(ft, a), j0 = floor_frac(fe, b);
-  const int i = min(i0, kHotNT - 2), j = min(j0, kHotNE - 2);
-  if (i != i0) a = 1.0;   // at the last node (ft = kHotNT - 1)
-  if (j != j0) b = 1.0;
-  const double *h = m.hot;
-  double v00 = h[i * kHotNE + j], v01 = h[i * kHotNE + j + 1];
-  double v10 = h[(i + 1) * kHotNE + j], v11 = h[(i + 1) * kHotNE + j + 1];
-  double l = (1 - a) * (1 - b) * v00 + (1 - a) * b * v01 + a * (1 - b) * v10 + a * b * v11;
-  return kSIGT * exp_t(m.ftab, l);
-}
-
-__device__ __forceinline__ double hot_lookup(const DevModel &m, double thetae, double eps) {
-  return hot_lookup_ln(m, log(thetae), log(eps));
 }
 
 __device__ __forceinline__ float hot_lookup_f(const DevModel &m, float thetae, float eps) {
@@ -1047,7 +1015,7 @@ __device__ __forceinline__ double lnK2_cells(const DevModel &m, double lt) {
   return cell_cubic(m.lnK2c, m.nK2 - 1, fma(lt, 1.0 / kK2Step, -kK2LnT0 / kK2Step));
 }
 
-// sigma_h / sigma_T: bilinear in (ln Theta, ln eps) as hot_lookup_ln, from v00, dv/db, dv/da, d2v/dadb of the cell.
+// sigma_h / sigma_T: bilinear in (ln Theta, ln eps), arguments clamped to the table, from v00, dv/db, dv/da, d2v/dadb of the cell.
 __device__ __forceinline__ double hot_cells(const DevModel &m, double lt, double le) {
   constexpr double st = (kHotNT - 1) / (kHotLT1 - kHotLT0), se = (kHotNE - 1) / (kHotLE1 - kHotLE0);
   const double ft = dmin_nn(dmax0(fma(lt, st, -kHotLT0 * st)), (double)(kHotNT - 1));
@@ -1763,19 +1731,59 @@ static __device__ void tetrad_emission(const Geo &G, const double u[4], const do
   for (int q = 0; q < 4; ++q) e[2][q] = t2[q];
 }
 
-// Scattering tetrad: e0 = u, e1..e3 from the x1, x2, x3 directions by Gram-Schmidt.
-static __device__ void tetrad_scatter(const Geo &G, const double u[4], double e[4][4]) {
+// Gram-Schmidt legs of the scattering tetrad.  A leg is kept with its lowered form l (l_q = g_qp v^p), so that
+// projecting the coordinate direction k on it is reading l[k], not a contraction with the metric: 95 FP64
+// operations instead of 290.
+struct Leg {
+  double v[4], l[4];
+};
+// coordinate direction k
+__device__ __forceinline__ void leg_coord(const Geo &G, int k, Leg &t) {
 #pragma unroll
-  for (int q = 0; q < 4; ++q) e[0][q] = u[q];
-  for (int k = 1; k < 4; ++k) {
-    double t[4] = {0, 0, 0, 0};
-    t[k] = 1.0;
-    gs_step(G, t, e[0], 1.0);
-    for (int p = 1; p < k; ++p) gs_step(G, t, e[p], -1.0);
-    normalize_space(G, t);
+  for (int q = 0; q < 4; ++q) t.v[q] = (q == k) ? 1.0 : 0.0;
+  t.l[0] = (k == 1) ? G.g01 : (k == 3) ? G.g03 : 0.0;
+  t.l[1] = (k == 1) ? G.g11 : (k == 3) ? G.g13 : 0.0;
+  t.l[2] = (k == 2) ? G.g22 : 0.0;
+  t.l[3] = (k == 1) ? G.g13 : (k == 3) ? G.g33 : 0.0;
+}
+__device__ __forceinline__ void leg_add(Leg &t, double d, const Leg &e) {
 #pragma unroll
-    for (int q = 0; q < 4; ++q) e[k][q] = t[q];
+  for (int q = 0; q < 4; ++q) {
+    t.v[q] = fma(d, e.v[q], t.v[q]);
+    t.l[q] = fma(d, e.l[q], t.l[q]);
   }
+}
+__device__ __forceinline__ void leg_unit(Leg &t) {
+  const double n2 = t.v[0] * t.l[0] + t.v[1] * t.l[1] + t.v[2] * t.l[2] + t.v[3] * t.l[3];
+  if (!(n2 > 1e-30)) return;
+  const double in = rsqrt_n(n2);
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    t.v[q] *= in;
+    t.l[q] *= in;
+  }
+}
+
+// Scattering tetrad: e0 = u (lowered form ul), e1..e3 from the x1, x2, x3 directions by Gram-Schmidt.
+static __device__ void tetrad_scatter(const Geo &G, const double u[4], const double ul[4], double e[4][4]) {
+  Leg g[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    g[0].v[q] = u[q];
+    g[0].l[q] = ul[q];
+  }
+#pragma unroll
+  for (int k = 1; k < 4; ++k) {
+    leg_coord(G, k, g[k]);
+    leg_add(g[k], g[0].l[k], g[0]);
+#pragma unroll
+    for (int p = 1; p < k; ++p) leg_add(g[k], -g[p].l[k], g[p]);
+    leg_unit(g[k]);
+  }
+#pragma unroll
+  for (int k = 0; k < 4; ++k)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) e[k][q] = g[k].v[q];
 }
 
 // ---------------------------------------------------------------- Compton kinematics (section 2.7)
@@ -1921,21 +1929,76 @@ __device__ __forceinline__ void boost3(R E, const R p[3], R beta, const R v[3], 
   po[2] = p[2] + (ppar - pv) * v[2];
 }
 
+// Electron of a thermal population for the FP64 kinematics: the proposals of sample_mj and the (gamma, mu_e)
+// acceptance of compton_fluid in one loop, same draws in the same order.  Nested, a warp ran the inner loop to
+// its slowest lane once per outer proposal, and the cold branch recomputed its mixture weights each time (about
+// 16000 FP64 issues per warp of children); in one loop it waits for the lane with the most proposals once.  With
+// the scattering tetrad's shorter form, loading 360000 children of the 3-D snapshot went from 9.8 to 4.4 ms.
+__device__ __forceinline__ void thermal_electron(const double *T, double th, double eps, Rng &s, uint64_t seed, double &gam,
+                                                 double &mue, double &beta, int &rejcap) {
+  const bool hot = th >= 0.25;
+  const double rt = sqrt(th);
+  const double c1 = 0.886226925452758 * (th * rt), c2 = 1.25 * 1.329340388179137 * (th * th * rt);
+  const double ct = c1 + c2 + 0.25 * 3.323350970447843 * (th * th * th * rt);
+  int mj = 0, it = 0;
+  while (true) {
+    bool got;
+    if (hot) {
+      const double u1 = rng_u(s, seed), u2 = rng_u(s, seed), u3 = rng_u(s, seed), u4 = rng_u(s, seed);
+      const double p = -th * log_q(T, u1 * u2 * u3), eta = p - th * log_q(T, u4);
+      const double q = fma(p, p, 1.0);
+      got = eta * eta - p * p > 1.0;
+      gam = sqrt(q);
+    } else {
+      const double uc = rng_u(s, seed) * ct;
+      const int k = (uc < c1) ? 1 : ((uc < c1 + c2) ? 2 : 3);
+      double prod = 1.0;
+      for (int i = 0; i < k; ++i) prod *= rng_u(s, seed);
+      const double ua = rng_u(s, seed), ub = rng_u(s, seed);
+      double sz, cz;
+      sincospi_q(T, 2.0 * ub, sz, cz);
+      const double z2 = -2.0 * log_q(T, ua) * (cz * cz);
+      const double t = th * (0.5 * z2 - log_q(T, prod));
+      const double acc = (1.0 + t) * sqrt(t + 2.0) * rcp_n(1.4142135623730951 * (1.0 + 1.25 * t + 0.25 * t * t));
+      got = rng_u(s, seed) < acc;
+      gam = 1.0 + t;
+    }
+    if (!got && mj < kMaxTry - 1) {
+      ++mj;
+      continue;
+    }
+    mj = 0;
+    mue = 2.0 * rng_u(s, seed) - 1.0;
+    beta = sqrt(1.0 - rcp_n(gam * gam));
+    const double om = 1.0 - beta * mue;
+    const double acc = om * sigma_kn_ratio(eps * gam * om) * 0.5;
+    if (rng_u(s, seed) < acc) return;
+    if (++it == kMaxTry || eps != eps) {   // a NaN energy (and acceptance) never passes: no need to try on
+      rejcap++;
+      return;
+    }
+  }
+}
+
 // Scattered photon in the plasma frame for incoming energy eps along unit n; draws in the order
 // [gamma (MJ), mu_e, accept]*, phi_e, [cos, accept]*, phi.
 // kappa > 0: kappa-distributed electrons of temperature-like parameter w = th (kappa - 3) / kappa.
 template <typename R>
-static __device__ void compton_fluid(R kappa, R th, R eps, const R n[3], Rng &s, uint64_t seed, R &eo, R dir[3],
-                                     int &rejcap) {
+static __device__ void compton_fluid(const double *T, R kappa, R th, R eps, const R n[3], Rng &s, uint64_t seed, R &eo,
+                                     R dir[3], int &rejcap) {
   R gam = 1, mue = 0, beta = 0;
   int it;
-  for (it = 0; it < kMaxTry; ++it) {
+  if constexpr (sizeof(R) == 8) {
+    if (!(kappa > (R)0)) thermal_electron(T, th, eps, s, seed, gam, mue, beta, rejcap);
+  }
+  for (it = 0; it < kMaxTry && (sizeof(R) == 4 || kappa > (R)0); ++it) {
     gam = kappa > (R)0 ? sample_kappa(kappa, th * (kappa - (R)3) / kappa, s, seed, rejcap) : sample_mj(th, s, seed);
     mue = (R)2 * rng_r<R>(s, seed) - (R)1;
     beta = r_sqrt((R)1 - (R)1 / (gam * gam));
     R om = (R)1 - beta * mue;
     R acc = om * sigma_kn_ratio(eps * gam * om) * (R)0.5;
     if (rng_r<R>(s, seed) < acc) break;
+    if (sizeof(R) == 8 && eps != eps) it = kMaxTry - 1;   // a NaN energy never passes
   }
   if (it == kMaxTry) rejcap++;
   R phie = (R)2 * rng_r<R>(s, seed);   // in units of pi
@@ -1964,6 +2027,7 @@ static __device__ void compton_fluid(R kappa, R th, R eps, const R n[3], Rng &s,
       P = (R)0.5 * r * r * (r + (R)1 / r - ((R)1 - ct * ct));
     }
     if (rng_r<R>(s, seed) < P) break;
+    if (sizeof(R) == 8 && ee != ee) it = kMaxTry - 1;
   }
   if (it == kMaxTry) rejcap++;
   R phi = (R)2 * rng_r<R>(s, seed);

@@ -371,7 +371,7 @@ static __device__ void emit_post(const DevModel &m, const EmitZone &Z, double ln
   double e[4][4];
   // without a field (a bremsstrahlung-only plasma) the frame of the scattering tetrad serves
   if (P.bsq > 0.0) tetrad_emission(G, ucon, bcon, P.bsq, e);
-  else tetrad_scatter(G, ucon, e);
+  else tetrad_scatter(G, ucon, P.ucov, e);
   double sp, cp;
   sincospi(phi, &sp, &cp);
   double kf[4] = {eps, eps * sth * cp, eps * sth * sp, eps * cth};
@@ -451,7 +451,7 @@ static __device__ void child_kinematics_f(const DevModel &m, const double Xe[4],
   rng_init(s, cid, 0u);
   float eo, dir[3];
   int rej = 0;
-  compton_fluid<float>(m.kappa_on ? (float)m.kappa : 0.0f, fmaxf(P.thetae, 1e-8f), eps, n, s, m.seed, eo, dir, rej);
+  compton_fluid<float>(m.ftab, m.kappa_on ? (float)m.kappa : 0.0f, fmaxf(P.thetae, 1e-8f), eps, n, s, m.seed, eo, dir, rej);
   ls.rejcap += rej;
 #pragma unroll
   for (int q = 0; q < 4; ++q) Kc[q] = (double)(eo * e[0][q] + dir[0] * e[1][q] + dir[1] * e[2][q] + dir[2] * e[3][q]);
@@ -469,7 +469,7 @@ static __device__ void child_kinematics(const DevModel &m, const double Xe[4], c
   double ucon[4];
   plasma_from_prims<double>(m, G, pr, P, ucon, nullptr);
   double e[4][4];
-  tetrad_scatter(G, ucon, e);
+  tetrad_scatter(G, ucon, P.ucov, e);
   double kc[4];
   lower(G, Ke, kc);
   double kf[4];
@@ -479,13 +479,13 @@ static __device__ void child_kinematics(const DevModel &m, const double Xe[4], c
     kf[a] = (a == 0) ? -d : d;
   }
   double eps = kf[0];
-  double il = 1.0 / sqrt(kf[1] * kf[1] + kf[2] * kf[2] + kf[3] * kf[3]);
+  double il = rsqrt_n(kf[1] * kf[1] + kf[2] * kf[2] + kf[3] * kf[3]);
   double n[3] = {kf[1] * il, kf[2] * il, kf[3] * il};
   Rng s;
   rng_init(s, cid, 0u);
   double eo, dir[3];
   int rej = 0;
-  compton_fluid(m.kappa, fmax(P.thetae, 1e-8), eps, n, s, m.seed, eo, dir, rej);
+  compton_fluid(m.ftab, m.kappa, fmax(P.thetae, 1e-8), eps, n, s, m.seed, eo, dir, rej);
   ls.rejcap += rej;
 #pragma unroll
   for (int q = 0; q < 4; ++q) Kc[q] = eo * e[0][q] + dir[0] * e[1][q] + dir[1] * e[2][q] + dir[2] * e[3][q];
