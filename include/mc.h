@@ -137,7 +137,8 @@ typedef struct mc_run_stats {
   int64_t n_steps_grid;  /* steps taken inside the radial extent of the grid (the rest free-stream) */
   int64_t n_iters_grid;  /* Verlet predictor passes of those steps */
   double init_ms, grid_ms, free_ms;   /* transport device time by phase: emission/initialisation,
-                                         in-grid push, free-streaming push */
+                                         in-grid push, free-streaming push (small generations run both in
+                                         one launch, counted as in-grid) */
   int32_t batch_min_blocks;  /* mc_run_batch: register-cap variant (minimum resident CTAs per SM) */
   int32_t batch_ctas;        /* mc_run_batch: persistent grid size in CTAs */
   int32_t batch_graph;       /* mc_run_batch: 1 if the run replayed a captured CUDA graph */

@@ -582,6 +582,23 @@ static double tune_next_scale(double s, int64_t carried, int64_t children, doubl
   return std::min(1e12, s * f);
 }
 
+// A generation (or a list handed back) of at most this many superphotons per warp of a full launch goes through
+// both phases in one launch.  Measured at 0 (never), 1, 2, 4, 8, 16 (ms a pass): the 64 x 32 sphere at N_s = 2000
+// 20.1, 17.7, 16.8, 16.7, 16.9, 16.7; the FP64 scattering sphere 91.7, 90.2, 90.5, 85.1, 84.8, 85.2; a 3-D torus at
+// N_s = 44000 38.9, 38.7, 37.7, 38.0, 39.4, 40.0 (more lanes of one warp in different phases).
+static const int64_t kSmallLanes = 4;
+static int push_small(mc_ctx *c, const DevModel &m, PushIO &pio, int prec, const int32_t *list, int64_t n, int64_t warps,
+                      int block, cudaStream_t st) {
+  pio.list_in = list;
+  pio.list_out = nullptr;
+  pio.n_in = n;
+  pio.lanes = (int)((n + warps - 1) / warps);
+  const int64_t per_cta = (int64_t)pio.lanes * (block / 32);
+  TIMED_LAUNCH(1, launch_push(m, pio, prec, 2, (int)((n + per_cta - 1) / per_cta), block, st));
+  if (c->cnt_host[CNT_ERR] & 1ull) return fail(c, MC_ERR_QUEUE_OVERFLOW, "scattered-superphoton queue overflow");
+  return MC_OK;
+}
+
 static int transport(mc_ctx *c, int64_t u0, int64_t u1, const int64_t *uid_list_dev, int64_t n_list, mc_log_rec *log_dev,
                      int64_t log_cap, uint64_t seed, cudaStream_t st, bool tune) {
   DevModel m = make_model(c);
@@ -591,8 +608,8 @@ static int transport(mc_ctx *c, int64_t u0, int64_t u1, const int64_t *uid_list_
   const bool tuning = tune && c->p.bias_target > 0.0;
   const int block = c->p.block ? c->p.block : 128;
   const int prec = c->p.precision;
-  int occ[2];
-  for (int ph = 0; ph < 2; ++ph) {
+  int occ[3];   // resident CTAs per SM of the in-grid, free-streaming and both-phase kernels
+  for (int ph = 0; ph < 3; ++ph) {
     occ[ph] = std::max(1, push_max_blocks_per_sm(prec, ph, block, m.a != 0.0 ? 1 : 0));
     if (c->p.ctas_per_sm > 0) occ[ph] = std::min(occ[ph], (int)c->p.ctas_per_sm);
   }
@@ -653,7 +670,20 @@ static int transport(mc_ctx *c, int64_t u0, int64_t u1, const int64_t *uid_list_
       int grid_init = (int)std::min<int64_t>((int64_t)c->sms * 4, (n_items + block - 1) / block);
       TIMED_LAUNCH(0, launch_init(m, iio, prec, grid_init, block, st));
       int64_t n_grid = (int64_t)c->cnt_host[CNT_L0], n_free = (int64_t)c->cnt_host[CNT_L1];
+      const int64_t warps = (int64_t)c->sms * occ[2] * (block / 32);
+      const auto small = [&](int64_t n) { return !use_sur && n <= kSmallLanes * warps; };
+      if (small(n_items)) {   // both phases in one launch, spread over the warps
+        rc = push_small(c, m, pio, prec, nullptr, n_items, warps, block, st);
+        if (rc) return rc;
+        n_grid = n_free = 0;
+      }
       while (n_grid > 0 || n_free > 0) {
+        if (n_grid > 0 && n_free == 0 && small(n_grid)) {   // the few that came back into the grid
+          rc = set_counter(c, CNT_NEXT, 0, st);
+          if (!rc) rc = push_small(c, m, pio, prec, c->list_grid, n_grid, warps, block, st);
+          if (rc) return rc;
+          n_grid = 0;
+        }
         if (n_grid > 0) {
           rc = set_counter(c, CNT_NEXT, 0, st);
           if (rc) return rc;

@@ -73,6 +73,7 @@ struct PushIO {
   unsigned long long *cnt;  // CNT_N counters
   mc_log_rec *log;
   int64_t log_cap;
+  int lanes;                // superphotons per warp (both-phase launches)
 };
 
 // tables (mc_tables.cu)
@@ -98,7 +99,7 @@ void launch_kappa_tables(double kappa, double *lnF, double *lnJ, double *lnA, do
 // prec: the precision form (MC_PREC_FP64, MC_PREC_MIXED or MC_PREC_SPLIT)
 int push_max_blocks_per_sm(int prec, int phase, int block, int kerr);
 void launch_init(const DevModel &m, const InitIO &io, int prec, int grid, int block, cudaStream_t st);
-// phase 0: superphotons inside the radial extent of the grid; 1: outside it
+// phase 0: superphotons inside the radial extent of the grid; 1: outside it; 2: both (slots 0 .. n_in - 1 of the pool)
 void launch_push(const DevModel &m, const PushIO &io, int prec, int phase, int grid, int block, cudaStream_t st);
 // in-grid push with the coefficient network (mixed or split form; 128-thread row groups)
 int push_sur_max_blocks_per_sm(int prec, int block, int smem, int kerr);

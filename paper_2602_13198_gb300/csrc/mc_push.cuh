@@ -925,6 +925,21 @@ __device__ __forceinline__ void load_ph(const Pool &P, int64_t i, PhT<S, W> &p) 
   p.raddr = nullptr;
 }
 
+// What save_ph and load_ph do to a state between phases, in registers: the double-float pairs normalised from their
+// sums, the relative weight through the absolute one (FP64 states pass unchanged).
+template <typename S, typename W>
+__device__ __forceinline__ void repack_ph(PhT<S, W> &p) {
+  if constexpr (std::is_same<S, df>::value) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      p.X[q] = from_d<S>(to_d(p.X[q]));
+      p.K[q] = from_d<S>(to_d(p.K[q]));
+      p.A[q] = from_d<S>(to_d(p.A[q]));
+    }
+  }
+  if constexpr (std::is_same<W, float>::value) p.w = (float)(abs_w(p) / p.wb);
+}
+
 // roulette threshold of model m: roulette_w * wb (relative weights: roulette_w)
 template <typename S, typename W>
 __device__ __forceinline__ void set_wthr(const DevModel &m, PhT<S, W> &p) {

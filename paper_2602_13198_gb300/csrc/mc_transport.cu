@@ -62,7 +62,9 @@ __global__ void __launch_bounds__(128) k_init(DevModel m, InitIO io) {
 
 // Persistent transport of one phase over io.list_in; PHASE 0 keeps superphotons while they are in
 // the grid, PHASE 1 while they are outside it.  A lane whose superphoton ends or changes phase is
-// refilled from the list (one atomic per warp).
+// refilled from the list (one atomic per warp).  PHASE 2 carries the listed superphotons (no list: slots 0 .. n_in - 1)
+// through both phases to their ends, io.lanes of them per warp: a small generation is bound by its longest
+// paths, one after another in every phase launch, and by the paths a warp's lanes take apart, not by throughput.
 template <int PREC, int PHASE, bool KERR>
 __device__ __forceinline__ void push_body(const DevModel &m, const PushIO &io) {
   const int lane = threadIdx.x & 31;
@@ -72,9 +74,11 @@ __device__ __forceinline__ void push_body(const DevModel &m, const PushIO &io) {
   int64_t slot = -1;
   bool live = false;
   bool exhausted = false;
+  bool grid_phase = true;                               // PHASE 2: where this lane's superphoton is
+  const bool use = PHASE != 2 || lane < io.lanes;
   while (true) {
     if (!exhausted) {
-      unsigned idle = __ballot_sync(0xffffffffu, !live);
+      unsigned idle = __ballot_sync(0xffffffffu, !live && use);
       if (idle) {
         int cnt = __popc(idle);
         int leader = __ffs(idle) - 1;
@@ -82,11 +86,12 @@ __device__ __forceinline__ void push_body(const DevModel &m, const PushIO &io) {
         if (lane == leader) base = atomicAdd(io.cnt + CNT_NEXT, (unsigned long long)cnt);
         base = __shfl_sync(0xffffffffu, base, leader);
         if (base + cnt >= (unsigned long long)io.n_in) exhausted = true;
-        if (!live) {
+        if (!live && use) {
           unsigned long long k = base + __popc(idle & ((1u << lane) - 1u));
           if (k < (unsigned long long)io.n_in) {
-            slot = io.list_in[k];
+            slot = (PHASE == 2 && !io.list_in) ? (int64_t)k : io.list_in[k];
             load_ph(io.pool, slot, p, m);
+            if (PHASE == 2) grid_phase = in_grid(m, p.X);
             live = true;
           }
         }
@@ -95,7 +100,23 @@ __device__ __forceinline__ void push_body(const DevModel &m, const PushIO &io) {
     if (!__any_sync(0xffffffffu, live)) break;
     if (live) {
       bool handoff;
-      if (PHASE == 0) {
+      if (PHASE == 2) {
+        handoff = false;
+        if (grid_phase) {
+          live = step<PREC, KERR, false>(m, io, p, ls);
+          if (live && !in_grid(m, p.X)) {
+            grid_phase = false;
+            repack_ph(p);
+          }
+        } else {
+          const int r = step_free<PREC, KERR>(m, io, p, ls);
+          live = (r != 1);
+          if (r == 2) {
+            grid_phase = true;
+            repack_ph(p);
+          }
+        }
+      } else if (PHASE == 0) {
         live = step<PREC, KERR, false>(m, io, p, ls);
         handoff = live && !in_grid(m, p.X);
       } else {
@@ -143,6 +164,12 @@ __global__ void __launch_bounds__(128, MC_MIXED_MINB) k_push_mixed(DevModel m, P
 template <int PHASE, bool KERR>
 __global__ void __launch_bounds__(128, MC_SPLIT_MINB) k_push_split(DevModel m, PushIO io) {
   push_body<2, PHASE, KERR>(m, io);
+}
+
+// Both phases for a small generation (no cap on registers: the resident warps are not what it waits for).
+template <int PREC, bool KERR>
+__global__ void __launch_bounds__(128, 1) k_push_small(DevModel m, PushIO io) {
+  push_body<PREC, 2, KERR>(m, io);
 }
 
 // Persistent in-grid push with the network.  Each 128-thread row group reaches its tensor-core
@@ -229,18 +256,25 @@ void launch_push_sur(const DevModel &m, const PushIO &io, const SurrogateView &s
   cudaLaunchKernel(sur_kernel(prec, m.a != 0.0), dim3(grid), dim3(128 * kTcGroupsMax), args, smem, st);
 }
 
-// Kernel of one launch configuration: precision form, phase and spin (general Kerr, or a = 0).
+// Kernel of one launch configuration: precision form, phase (2: both) and spin (general Kerr, or a = 0).
+template <int PREC>
+static const void *small_kernel(bool kerr) {
+  return kerr ? (const void *)k_push_small<PREC, true> : (const void *)k_push_small<PREC, false>;
+}
 template <int PHASE>
-static const void *push_kernel(int prec, bool kerr) {
+static const void *phase_kernel(int prec, bool kerr) {
   if (prec == 1) return kerr ? (const void *)k_push_mixed<PHASE, true> : (const void *)k_push_mixed<PHASE, false>;
   if (prec == 2) return kerr ? (const void *)k_push_split<PHASE, true> : (const void *)k_push_split<PHASE, false>;
   return kerr ? (const void *)k_push_fp64<PHASE, true> : (const void *)k_push_fp64<PHASE, false>;
 }
+static const void *push_kernel(int prec, int phase, bool kerr) {
+  if (phase == 2) return prec == 1 ? small_kernel<1>(kerr) : prec == 2 ? small_kernel<2>(kerr) : small_kernel<0>(kerr);
+  return phase == 0 ? phase_kernel<0>(prec, kerr) : phase_kernel<1>(prec, kerr);
+}
 
 int push_max_blocks_per_sm(int prec, int phase, int block, int kerr) {
   int n = 0;
-  const void *k = phase == 0 ? push_kernel<0>(prec, kerr != 0) : push_kernel<1>(prec, kerr != 0);
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, block, 0);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, push_kernel(prec, phase, kerr != 0), block, 0);
   return n;
 }
 
@@ -258,10 +292,8 @@ void launch_init(const DevModel &m, const InitIO &io, int prec, int grid, int bl
 
 // a = 0 takes the Schwarzschild form of the metric and of the geodesic acceleration.
 void launch_push(const DevModel &m, const PushIO &io, int prec, int phase, int grid, int block, cudaStream_t st) {
-  const bool kerr = m.a != 0.0;
   void *args[] = {(void *)&m, (void *)&io};
-  const void *k = phase == 0 ? push_kernel<0>(prec, kerr) : push_kernel<1>(prec, kerr);
-  cudaLaunchKernel(k, dim3(grid), dim3(block), args, 0, st);
+  cudaLaunchKernel(push_kernel(prec, phase, m.a != 0.0), dim3(grid), dim3(block), args, 0, st);
 }
 
 }  // namespace mcgb
