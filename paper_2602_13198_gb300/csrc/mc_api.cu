@@ -163,6 +163,7 @@ DevModel make_model(const mc_ctx *c) {
   m.kapA = c->kapA;
   m.kapI = c->kapI;
   m.kapH = c->kapH;
+  m.kap_w = p.kappa > 0.0 ? (p.kappa - 3.0) / p.kappa : 0.0;
   m.gam2 = 2.0 * (p.gam - 1.0);
   m.cthe = (kMP / kME) * (p.gam - 1.0);
   m.hCcoef = 0.5 * m.Ccoef;
@@ -888,7 +889,7 @@ int mc_get_bias_scales(mc_ctx *c, double *scales, int n) {
 }
 
 int mc_selftest_math(int which, const double *x, double *y, double *ref, int64_t n) {
-  if (which < 0 || which > 18 || n < 0 || (n > 0 && (!x || !y || !ref))) return fail(nullptr, MC_ERR_INVALID_ARG, "bad argument");
+  if (which < 0 || which > 19 || n < 0 || (n > 0 && (!x || !y || !ref))) return fail(nullptr, MC_ERR_INVALID_ARG, "bad argument");
   int ndev = 0;
   if (cudaGetDeviceCount(&ndev) != cudaSuccess || ndev < 1) {
     cudaGetLastError();

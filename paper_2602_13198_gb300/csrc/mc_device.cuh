@@ -339,6 +339,7 @@ struct DevModel {
   int brems;              // thermal bremsstrahlung on
   df dmass, da, dx1_0, dx1_hi, dr_record, dr_capture;   // double-float splits for the mixed geodesic
   df dpi2hh, dhh_pi, dd2th;   // pi (1 - h), (1 - h) / (2 pi), -2 pi^2 (1 - h): the theta map in double-float
+  double kap_w;                // (kappa - 3) / kappa
   double gam2, cthe, hCcoef;   // 2 (gam - 1), (m_p / m_e) (gam - 1), Ccoef / 2
   double a2, twoa, M2, pi2hh, hh_pi2, d2th2;   // a^2, 2 a, 2 M and the theta map's pi (1-h), (1-h) / pi, -4 pi^2 (1-h)
   const df *dtab;             // double-float function table (kDfTabN entries)
@@ -1055,29 +1056,42 @@ __device__ __forceinline__ double kap_interp(const double *t, double lx, double 
   double l = (1 - a) * (1 - b) * r[0] + (1 - a) * b * r[1] + a * (1 - b) * r[kKapNW] + a * b * r[kKapNW + 1];
   return exp(l);
 }
+// The same for the transport: index coordinates clamped on their bit patterns, three lerps, the table-driven
+// logarithm and exponential, reciprocals from the hardware's seeds.  The library forms and their divisions held the
+// FP64 pipe of the split form for 64 of 269 ms (kappa torus with bremsstrahlung, 97 x 49, N_s = 3e5: 205 ms now).
+__device__ __forceinline__ double bilerp(const double *r, int stride, double a, double b) {
+  const double v0 = fma(b, r[1] - r[0], r[0]), v1 = fma(b, r[stride + 1] - r[stride], r[stride]);
+  return fma(a, v1 - v0, v0);
+}
+__device__ __forceinline__ int clamp_split(double f, int n, double &frac) {   // cell and fraction of f kept within [0, n - 1]
+  const int i0 = floor_frac(dmin_nn(dmax0(f), (double)(n - 1)), frac), i = min(i0, n - 2);
+  if (i != i0) frac = 1.0;
+  return i;
+}
 
-// nu alpha_nu of the kappa population at angle sth to the field
-__device__ __forceinline__ double kappa_nu_alpha(const DevModel &m, double ne, double thetae, double B, double sth,
-                                                 double nu) {
-  const double lx = log(nu / (kNuB1 * B * sth)), lw = log(thetae * (m.kappa - 3.0) / m.kappa);
+// nu alpha_nu of the kappa population at angle sth to the field; lw = ln w
+__device__ __forceinline__ double kappa_nu_alpha(const DevModel &m, double ne, double B, double sth, double nu, double lw) {
+  constexpr double sx = (kKapNX - 1) / (kKapLX1 - kKapLX0), sw = (kKapNW - 1) / (kKapLW1 - kKapLW0);
   constexpr double kCa = kCL * kCL / (8.0 * kPI) * kKapCj / (kME * kCL * kCL);
-  return kCa * ne * B * sth * kap_interp(m.kapA, lx, lw) / nu;
+  const double Bs = B * sth;
+  const double lx = log_q(m.ftab, nu * rcp_n(kNuB1 * Bs));
+  double fa, fb;
+  const int i = clamp_split(fma(lx, sx, -kKapLX0 * sx), kKapNX, fa), j = clamp_split(fma(lw, sw, -kKapLW0 * sw), kKapNW, fb);
+  return (kCa * ne) * Bs * exp_q(m.ftab, bilerp(m.kapA + i * kKapNW + j, kKapNW, fa, fb)) * rcp_n(nu);
 }
 
 // Hot cross-section of the kappa population, bilinear in (ln w, ln eps) on the kappa w grid and the
 // thermal table's eps grid (clamped to both)
-__device__ __forceinline__ double kap_hot_lookup(const DevModel &m, double thetae, double eps) {
+__device__ __forceinline__ double kap_hot_lookup(const DevModel &m, double lw, double eps) {
   constexpr double sw = (kKapNW - 1) / (kKapLW1 - kKapLW0), se = (kHotNE - 1) / (kHotLE1 - kHotLE0);
-  double fw = (log(fmax(thetae, 1e-300) * (m.kappa - 3.0) / m.kappa) - kKapLW0) * sw;
-  double fe = (log(eps) - kHotLE0) * se;
-  fw = fmin(fmax(fw, 0.0), (double)(kKapNW - 1));
-  fe = fmin(fmax(fe, 0.0), (double)(kHotNE - 1));
-  int i = min((int)fw, kKapNW - 2), j = min((int)fe, kHotNE - 2);
-  double a = fw - i, b = fe - j;
-  const double *h = m.kapH;
-  double v00 = h[i * kHotNE + j], v01 = h[i * kHotNE + j + 1];
-  double v10 = h[(i + 1) * kHotNE + j], v11 = h[(i + 1) * kHotNE + j + 1];
-  return kSIGT * exp((1 - a) * (1 - b) * v00 + (1 - a) * b * v01 + a * (1 - b) * v10 + a * b * v11);
+  double fa, fb;
+  const int i = clamp_split(fma(lw, sw, -kKapLW0 * sw), kKapNW, fa);
+  const int j = clamp_split(fma(log_q(m.ftab, eps), se, -kHotLE0 * se), kHotNE, fb);
+  return kSIGT * exp_q(m.ftab, bilerp(m.kapH + i * kHotNE + j, kHotNE, fa, fb));
+}
+// ln w of the kappa population at Theta_e
+__device__ __forceinline__ double kap_lnw(const DevModel &m, double thetae) {
+  return log_q(m.ftab, dmax_nn(thetae, 1e-300) * m.kap_w);
 }
 
 // ---------------------------------------------------------------- bremsstrahlung (future work in section 6)
@@ -1098,11 +1112,30 @@ __device__ __forceinline__ double brems_q(double ne, double th) {
   return ne * ne * kAlphaF * kMc2 * kCL * (1.25 * kSIGT * fei + kRe * kRe * fee);
 }
 
+// The rate for the transport (same fits): powers and logarithms from the tables.
+__device__ __forceinline__ double brems_q_t(const double *T, double ne, double th) {
+  constexpr double kAlphaF = 7.2973525693e-3, kRe = 2.8179403262e-13, kMc2 = kME * kCL * kCL;
+  constexpr double kRt2Pi3 = 0.25397454373696387;   // sqrt(2 / pi^3)
+  constexpr double kFee = 20.0 / (9.0 * 1.7724538509055161) * (44.0 - 3.0 * kPI * kPI);
+  double fei, fee;
+  if (th < 1.0) {
+    const double rt = th * rsqrt(th);
+    fei = (4.0 * kRt2Pi3 * rt) * fma(1.781, exp_q(T, 1.34 * log_q(T, th)), 1.0);
+    fee = kFee * th * rt * (1.0 + 1.1 * th + th * th - 1.25 * th * th * rt);
+  } else {
+    fei = 9.0 * th / (2.0 * kPI) * (log_q(T, 1.123 * th + 0.48) + 1.5);
+    fee = 24.0 * th * (log_q(T, 1.1232 * th) + 1.28);
+  }
+  return ne * ne * (kAlphaF * kMc2 * kCL) * (1.25 * kSIGT * fei + kRe * kRe * fee);
+}
+
 // nu alpha_nu = nu j_nu / B_nu = q c^2 (1 - exp(-h nu / k T)) / (8 pi k T nu^2)
-__device__ __forceinline__ double brems_nu_alpha(double ne, double th, double nu) {
+__device__ __forceinline__ double brems_nu_alpha(const DevModel &m, double ne, double th, double nu) {
   if (!(ne > 0.0 && th > 0.0)) return 0.0;
-  const double kt = th * kME * kCL * kCL;
-  return brems_q(ne, th) * kCL * kCL * (-expm1(-kHPL * nu / kt)) / (8.0 * kPI * kt * nu * nu);
+  const double x = kHPL * nu / (th * kME * kCL * kCL);
+  // -expm1(-x) = expm1(x) / (1 + expm1(x)); beyond x = 40 it is 1
+  const double e = x < 40.0 ? expm1_q(m.ftab, x) : 0.0, f = x < 40.0 ? e / (1.0 + e) : 1.0;
+  return brems_q_t(m.ftab, ne, th) * (kCL * kCL / (8.0 * kPI * kME * kCL * kCL)) * f / (th * nu * nu);
 }
 
 // int dOmega j_nu of zone z at weight-table node j: synchrotron (pref F(nu/nu_c); 0 when the zone
@@ -1479,7 +1512,7 @@ __device__ __forceinline__ void coefficients64(const DevModel &m, const Point &G
     if (__double_as_longlong(s2) > 0) {   // |cos| < 1
       const double rs = rsqrt_n(s2);
       if (m.kappa_on) {
-        c.ana = kappa_nu_alpha(m, ne, th, B, s2 * rs, nu);
+        c.ana = kappa_nu_alpha(m, ne, B, s2 * rs, nu, kap_lnw(m, th));
       } else {
         constexpr double kNus = (2.0 / 9.0) * (kEE / (2.0 * kPI * kME * kCL));   // nu_s / (B Theta^2 sin)
         const double nus = (kNus * B) * (th * th) * (s2 * rs);
@@ -1498,9 +1531,9 @@ __device__ __forceinline__ void coefficients64(const DevModel &m, const Point &G
       }
     }
   }
-  if (m.brems) c.ana += brems_nu_alpha(ne, th, nu);
+  if (m.brems) c.ana += brems_nu_alpha(m, ne, th, nu);
   if (want_s)
-    c.ans = (nu * ne) * (m.kappa_on ? kap_hot_lookup(m, th, eps) : kSIGT * hot_cells(m, lt, log_q(m.ftab, eps)));
+    c.ans = (nu * ne) * (m.kappa_on ? kap_hot_lookup(m, kap_lnw(m, th), eps) : kSIGT * hot_cells(m, lt, log_q(m.ftab, eps)));
 }
 
 // Mixed precision: the same quantities with FP32 plasma state and coefficient arithmetic.
@@ -1547,17 +1580,17 @@ __device__ __forceinline__ void coefficients32(const DevModel &m, const GeoT<S> 
     c.ana = (W)0;
     if (P.thetae >= m.fthetae_min && P.B > 0.0f && P.bsq > 0.0f) {
       double kb = to_d(K[0]) * P.bcov[0] + to_d(K[1]) * P.bcov[1] + to_d(K[2]) * P.bcov[2] + to_d(K[3]) * P.bcov[3];
-      double cth = fmin(1.0, fmax(-1.0, kb / ((double)eps * sqrt((double)P.bsq))));
-      double s2 = 1.0 - cth * cth;
-      if (s2 > 0.0)
-        c.ana = (W)kappa_nu_alpha(m, (double)P.ne, (double)P.thetae, (double)P.B, sqrt(s2), (double)nu9 * 1e9);
+      const double cth = kb * (rsqrt_n((double)P.bsq) * rcp_n((double)eps));
+      const double s2 = fma(-cth, cth, 1.0);
+      if (s2 > 0.0)   // |cos| < 1
+        c.ana = (W)kappa_nu_alpha(m, (double)P.ne, (double)P.B, s2 * rsqrt_n(s2), (double)nu9 * 1e9, kap_lnw(m, (double)P.thetae));
     }
   }
   // bremsstrahlung absorption in FP64 (n_e^2 leaves the FP32 range in dense plasma)
-  if (m.brems) c.ana = (W)((double)c.ana + brems_nu_alpha((double)P.ne, (double)P.thetae, (double)nu9 * 1e9));
+  if (m.brems) c.ana = (W)((double)c.ana + brems_nu_alpha(m, (double)P.ne, (double)P.thetae, (double)nu9 * 1e9));
   if (want_s) {
     if (m.kappa_on) {
-      c.ans = (W)((double)nu9 * 1e9 * (double)P.ne * kap_hot_lookup(m, (double)P.thetae, (double)eps));
+      c.ans = (W)((double)nu9 * 1e9 * (double)P.ne * kap_hot_lookup(m, kap_lnw(m, (double)P.thetae), (double)eps));
     } else {
       float sh = hot_lookup_f(m, fmaxf(P.thetae, 1e-30f), eps);
       c.ans = (W)(nu9 * P.ne * (sh * 1e9f));

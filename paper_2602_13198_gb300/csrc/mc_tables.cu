@@ -681,6 +681,11 @@ __global__ void k_selftest_math(int which, const double *x, double *y, double *r
     ref[i] = rsqrt(v);
     return;
   }
+  if (which == 19) {
+    y[i] = brems_q_t(F, 1.0, v);
+    ref[i] = brems_q(1.0, v);
+    return;
+  }
   if (which == 8 || which == 9) {
     double s, c, rs, rc;
     sincospi_t(F, v, s, c);

@@ -74,3 +74,11 @@ def test_reciprocals(which):
     x = np.concatenate([10.0 ** RNG.uniform(-290, 290, 300000), RNG.uniform(0.5, 4.0, 200000), 2.0 ** np.arange(-100, 101)])
     y, ref = both(which, x)
     assert rel(y, ref) <= 2 * ULP
+
+
+def test_brems_rate():
+    x = np.concatenate([10.0 ** RNG.uniform(-6, 3, 200000), [1.0, np.nextafter(1.0, 0.0), 1e-30, 1e-300, 1e6]])
+    y, ref = both(19, x)
+    # all terms are positive: some ten roundings, and 3 ulp of an exponent of at most 1.34 |ln x| in a term
+    # that x^1.34 makes small
+    assert rel(y, ref) <= 20 * ULP
