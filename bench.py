@@ -58,6 +58,9 @@ SURVEY = ("batched parameter survey: 64 synthetic 2-D Fishbone-Moncrief tori dra
 # Algorithmic operation counts (add/mul/div/sqrt = 1, FMA = 2, each transcendental = 1), itemised
 # from the formulas each kernel form evaluates.  The spin form is the one the library launches: the
 # Schwarzschild form (a = 0) leaves out the terms that vanish at a = 0; 3-D grids blend 8 corners.
+# The metric and acceleration are counted by components, a fixed unit of work per step; the FP64 geodesic
+# reaches the same values from the Kerr-Schild form with about a quarter of the operations, so its rate in
+# this unit can pass what the pipe executes.
 OPS_STEPSIZE = 10          # 1 / (|k1|/d1 + |k2|/d2 + |k3|/d3) in one division
 OPS_POSITION = 28          # x_{n+1} = x_n + k dl + dl^2/2 a (4 components) and the predictor start
 OPS_METRIC = {"kerr": 135, "schw": 59}      # metric, inverse and x1/x2 derivatives at x_{n+1}
@@ -103,7 +106,7 @@ DF_FLOPS_PER_OP = 9.0
 # (dram__bytes_read.sum + dram__bytes_write.sum of one launch / superphotons it carried); traffic grows
 # in proportion to the superphotons a launch carries.  Keyed by (workload, form); re-taken whenever
 # the kernel changes (profiles/ holds the summaries).
-TRAFFIC_B_PER_PH = {("c4", "fp64"): 6641.8}
+TRAFFIC_B_PER_PH = {("c4", "fp64"): 6426.0}
 # ncu-measured pipe utilisation of the double-float in-grid kernel (a full capture of its first launch
 # on the 3-D snapshot at N_s = 4e6): FP32 and FP64 pipes busy, issue active.
 NCU_MIXED_FP32_PIPE = {"in_grid_fp32": 0.257, "in_grid_fp64": 0.159, "issue_active": 0.370,
@@ -229,14 +232,16 @@ def sum_stats(stats):
 
 def fp64_roofline(st, spin, dim, fp64_peak, kernel, traffic_per_ph=None, hbm_peak=None, fp32_peak=None):
     """In-grid FP64 kernel against the measured FP64 FMA peak: achieved = the itemised count of the
-    form that ran x the step, pass and event counters / the in-grid phase's event-timed duration."""
+    form that ran, by metric components, x the step, pass and event counters / the in-grid phase's event-timed
+    duration: work done per second, not instructions executed."""
     t_grid = st["grid_ms"] / 1e3
     ops = (ops_grid_step(spin, dim) * st["n_steps_grid"] + ops_pass(spin) * st["n_iters_grid"]
            + OPS_EVENT * st["n_events"])
     ach = ops / t_grid
     r = {"bound": "alu", "achieved": ach / 1e12, "peak": fp64_peak / 1e12, "unit": "TFLOP/s", "frac": ach / fp64_peak,
          "traffic": None, "kernel": kernel,
-         "count": {"spin_form": spin, "grid_dim": dim, "ops_per_in_grid_step": ops_grid_step(spin, dim),
+         "count": {"basis": "component form of the metric; the kernel's Kerr-Schild form executes fewer",
+                   "spin_form": spin, "grid_dim": dim, "ops_per_in_grid_step": ops_grid_step(spin, dim),
                    "ops_per_predictor_pass": ops_pass(spin), "ops_per_event": OPS_EVENT,
                    "in_grid_steps": st["n_steps_grid"], "predictor_passes": st["n_iters_grid"], "events": st["n_events"]},
          "peak_source": "measured: project FP64 FMA-chain microbenchmark on this GPU (mc_fma_peak)",
