@@ -51,11 +51,6 @@ __device__ __forceinline__ double abs_w(const PhT<S, W> &p) {
   else return p.w;
 }
 
-// weight relative to the birth weight.  A child born behind some 700 optical depths has a birth weight of 0 (about one
-// in fifty on the scattering sphere at tau = 0.1); its relative weight is 0 too, so that it ends as absorbed at
-// its first test and the children of its first step weigh 0, as in FP64, instead of 0/0.
-__device__ __forceinline__ float rel_w(double w, double wb) { return wb > 0.0 ? (float)(w / wb) : 0.0f; }
-
 struct LocalStats {
   unsigned long long emit, child, rec, abs, capt, maxst, steps, iters, nonconv, roul, rejcap, events, gsteps, giters;
 };
@@ -121,7 +116,10 @@ static __device__ void init_transport(const DevModel &m, Ph &p) {
   }
   p.nsteps = 0;
   p.nev = 0;
-  p.wb = p.w;
+  // A child born behind some 700 optical depths weighs 0 (about one in fifty on the scattering sphere at tau = 0.1); its
+  // relative weight is then 0 of 1, so that it ends as absorbed at its first test and the children of its first
+  // step weigh 0, as in FP64, instead of 0/0.
+  p.wb = p.w > 0.0 ? p.w : 1.0;
 }
 
 // Emission of primary uid (section 2.3) at the centre of its zone: frequency proposed from the
@@ -915,7 +913,7 @@ __device__ __forceinline__ void load_ph(const Pool &P, int64_t i, PhT<S, W> &p) 
     p.A[q] = from_d<S>(P.A[q][i]);
   }
   p.wb = P.wb[i];
-  if constexpr (std::is_same<W, float>::value) p.w = rel_w(P.w[i], p.wb);
+  if constexpr (std::is_same<W, float>::value) p.w = (float)(P.w[i] / p.wb);
   else p.w = P.w[i];
   p.ana = (W)P.ana[i];
   p.ans = (W)P.ans[i];
@@ -942,7 +940,7 @@ __device__ __forceinline__ void repack_ph(PhT<S, W> &p) {
       p.A[q] = from_d<S>(to_d(p.A[q]));
     }
   }
-  if constexpr (std::is_same<W, float>::value) p.w = rel_w(abs_w(p), p.wb);
+  if constexpr (std::is_same<W, float>::value) p.w = (float)(abs_w(p) / p.wb);
 }
 
 // roulette threshold of model m: roulette_w * wb (relative weights: roulette_w)
