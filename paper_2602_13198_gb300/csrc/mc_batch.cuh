@@ -114,14 +114,14 @@ __device__ void batch_phase(const DevModel *sm, const BatchIO &b, const PushIO &
       }
       float in[3] = {0.0f, 0.0f, 0.0f}, out[3];
       if (live) {
-        step_sur_a<kPointForm<PREC, true, true>>(sm[p.model], p, sc, ls);
+        step_sur_a<kGeoForm<PREC, true, true>>(sm[p.model], p, sc, ls);
         in[0] = sc.a.in[0];
         in[1] = sc.a.in[1];
         in[2] = sc.a.in[2];
       }
       tc_mlp_eval(T, in, out);
       if (live) {
-        live = step_sur_b<PREC, kPointForm<PREC, true, true>>(sm[p.model], io, p, sc, out, ls);
+        live = step_sur_b<PREC, kGeoForm<PREC, true, true>>(sm[p.model], io, p, sc, out, ls);
         if (live && !in_grid(sm[p.model], p.X)) {
           save_ph(b.pool, slot, p);
           list_out[atomicAdd(out_cnt, 1ull)] = (int32_t)slot;

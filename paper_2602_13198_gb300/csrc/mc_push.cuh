@@ -56,13 +56,15 @@ struct LocalStats {
 };
 
 
-// Geometry of a geodesic step: POINT, the point's Kerr-Schild factors (FP64); otherwise the metric's components
-// and derivatives, in double-float or, in the split form's in-grid steps where a = 0 can occur (single models
-// with a = 0, and batches), in FP64: that form narrows the components to FP32 by truncation, and
-// g_t1 = f r = 2 M exactly at a = 0, so a last-bit difference in FP64 is a whole FP32 step (6e-8) in the
-// coefficients, which moved some spectra by 4e-9.
+// Geometry of a geodesic step: the point's Kerr-Schild factors (kGeoPoint, FP64), or the metric's components
+// and derivatives (kGeoComp): in double-float and in the split form's in-grid steps at a = 0.  The split form narrows
+// the components to FP32 by truncation, and g_t1 = f r = 2 M exactly at a = 0, so a last-bit difference in FP64
+// is a whole FP32 step (6e-8) there in the coefficients, which moved some spectra by 4e-9.  A batch of split models
+// holds both kinds: each superphoton takes the form of its own model (kGeoModel), so that the batch follows the
+// same arithmetic as the model's own run (16 models, N_s up to 3e5: 129 ms, 143 with components for all).
+enum GeoForm { kGeoComp, kGeoPoint, kGeoModel };
 template <int PREC, bool KERR, bool BATCH>
-constexpr bool kPointForm = PREC == 0 || (PREC == 2 && KERR && !BATCH);
+constexpr GeoForm kGeoForm = PREC == 0 ? kGeoPoint : PREC == 1 ? kGeoComp : BATCH ? kGeoModel : KERR ? kGeoPoint : kGeoComp;
 template <bool POINT, typename S> struct GeomOf { using T = GeoT<S>; };
 template <> struct GeomOf<true, double> { using T = Point; };
 template <bool KERR>
@@ -79,6 +81,15 @@ __device__ __forceinline__ Geo geo_of(const DevModel &m, const Point &P) {
 }
 template <bool KERR, typename S>
 __device__ __forceinline__ const GeoT<S> &geo_of(const DevModel &, const GeoT<S> &G) { return G; }
+__device__ __forceinline__ void geom_by_model(const DevModel &m, double x1, double x2, Geo &G) {
+  if (m.a != 0.0) {
+    Point P;
+    point_eval<true>(m, x1, x2, P);
+    metric_of<true>(m, P, G);
+  } else {
+    metric_eval<true, true>(m, x1, x2, G);
+  }
+}
 // -k_t and cos(theta): k_t = -k^t + f L with L = k^t + r k^1 - a sin^2 k^phi
 template <bool KERR>
 __device__ __forceinline__ double energy_at_infinity(const Point &G, const double K[4], double &cth) {
@@ -791,32 +802,56 @@ __device__ __forceinline__ void verlet_loop(const DevModel &m, const GT &G, cons
   }
 }
 
-// One geodesic step with absorption, scattering and the termination tests; false when finished.
-template <int PREC, bool KERR, bool BATCH>
-static __device__ bool step(const DevModel &m, const PushIO &io, PhF<PREC> &p, LocalStats &ls) {
-  using S = typename Form<PREC>::S;
-  using W = typename Form<PREC>::W;
-  constexpr bool POINT = kPointForm<PREC, KERR, BATCH>;
-  const bool scat = m.scatter && p.nsc < m.n_sc_max;
-  const S dl = stepsize<POINT>(m, p.X, p.K);
+// Geodesic part of an in-grid step: step size, position, geometry G there, wavevector and acceleration.  X0, K0: the
+// step's start.
+template <bool KERR, bool POINT, typename S, typename W>
+__device__ __forceinline__ void move(const DevModel &m, PhT<S, W> &p, S X0[4], S K0[4], S &dl,
+                                     typename GeomOf<POINT, S>::T &G, int &it, bool &conv) {
+  dl = stepsize<POINT>(m, p.X, p.K);
   const double hd = half_step(dl);
-  S X0[4], K0[4], An[4], Kn[4];
+  S An[4], Kn[4];
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
     X0[q] = p.X[q];
     K0[q] = p.K[q];
     p.X[q] = verlet_x<POINT>(X0[q], K0[q], p.A[q], dl, hd);
   }
-  typename GeomOf<POINT, S>::T G;
   geom_eval<KERR>(m, p.X[1], p.X[2], G);
-  int it;
-  bool conv;
   verlet_loop<KERR, POINT>(m, G, K0, p.A, dl, hd, Kn, An, it, conv);
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
     p.K[q] = Kn[q];
     p.A[q] = An[q];
   }
+}
+
+// The same in the form of the superphoton's own model (split form in a batch); G as components.  SCHW: models with
+// a = 0 take the a = 0 form, as their own run does.
+template <bool SCHW, typename W>
+__device__ __forceinline__ void move_by_model(const DevModel &m, PhT<double, W> &p, double X0[4], double K0[4], double &dl,
+                                              Geo &G, int &it, bool &conv) {
+  if (m.a != 0.0) {
+    Point P;
+    move<true, true>(m, p, X0, K0, dl, P, it, conv);
+    metric_of<true>(m, P, G);
+  } else {
+    move<!SCHW, false>(m, p, X0, K0, dl, G, it, conv);
+  }
+}
+
+// One geodesic step with absorption, scattering and the termination tests; false when finished.
+template <int PREC, bool KERR, bool BATCH>
+static __device__ bool step(const DevModel &m, const PushIO &io, PhF<PREC> &p, LocalStats &ls) {
+  using S = typename Form<PREC>::S;
+  using W = typename Form<PREC>::W;
+  constexpr GeoForm F = kGeoForm<PREC, KERR, BATCH>;
+  const bool scat = m.scatter && p.nsc < m.n_sc_max;
+  S X0[4], K0[4], dl;
+  typename GeomOf<F == kGeoPoint, S>::T G;
+  int it;
+  bool conv;
+  if constexpr (F == kGeoModel) move_by_model<true>(m, p, X0, K0, dl, G, it, conv);
+  else move<KERR, F == kGeoPoint>(m, p, X0, K0, dl, G, it, conv);
   ls.iters += it;
   ls.giters += it;
   ls.gsteps++;
@@ -970,27 +1005,14 @@ struct SurCarry {
   CoefA a;
 };
 
-template <bool POINT, typename S, typename W>
+template <GeoForm F, typename S, typename W>
 static __device__ void step_sur_a(const DevModel &m, PhT<S, W> &p, SurCarry<S> &sc, LocalStats &ls) {
-  const S dl = stepsize<POINT>(m, p.X, p.K);
-  const double hd = half_step(dl);
-  S An[4], Kn[4];
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    sc.X0[q] = p.X[q];
-    sc.K0[q] = p.K[q];
-    p.X[q] = verlet_x<POINT>(sc.X0[q], sc.K0[q], p.A[q], dl, hd);
-  }
-  typename GeomOf<POINT, S>::T G;
-  geom_eval<true>(m, p.X[1], p.X[2], G);
+  typename GeomOf<F == kGeoPoint, S>::T G;
+  S dl;
   int it;
   bool conv;
-  verlet_loop<true, POINT>(m, G, sc.K0, p.A, dl, hd, Kn, An, it, conv);
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    p.K[q] = Kn[q];
-    p.A[q] = An[q];
-  }
+  if constexpr (F == kGeoModel) move_by_model<false>(m, p, sc.X0, sc.K0, dl, G, it, conv);
+  else move<true, F == kGeoPoint>(m, p, sc.X0, sc.K0, dl, G, it, conv);
   ls.iters += it;
   ls.giters += it;
   ls.gsteps++;
@@ -1003,7 +1025,7 @@ static __device__ void step_sur_a(const DevModel &m, PhT<S, W> &p, SurCarry<S> &
   coefficients32_a(m, geo_of<true>(m, G), p.X, p.K, sc.a);
 }
 
-template <int PREC, bool POINT>
+template <int PREC, GeoForm F>
 static __device__ bool step_sur_b(const DevModel &m, const PushIO &io, PhF<PREC> &p,
                                   const SurCarry<typename Form<PREC>::S> &sc, const float out[3], LocalStats &ls) {
   using W = typename Form<PREC>::W;
@@ -1011,8 +1033,11 @@ static __device__ bool step_sur_b(const DevModel &m, const PushIO &io, PhF<PREC>
   CoefT<W> c;
   coefficients32_b(m, sc.a, out, scat, c);
   absorb_scatter(m, io, p, sc.X0, sc.K0, sc.dl, c, scat, ls);
-  typename GeomOf<POINT, typename Form<PREC>::S>::T G;   // read only by the recording (sc.term == 1)
-  if (sc.term == 1) geom_eval<true>(m, p.X[1], p.X[2], G);
+  typename GeomOf<F == kGeoPoint, typename Form<PREC>::S>::T G;   // read only by the recording (sc.term == 1)
+  if (sc.term == 1) {
+    if constexpr (F == kGeoModel) geom_by_model(m, p.X[1], p.X[2], G);
+    else geom_eval<true>(m, p.X[1], p.X[2], G);
+  }
   return terminate<true>(m, io, G, p, sc.term, ls) == 0;
 }
 

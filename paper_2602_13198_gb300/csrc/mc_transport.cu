@@ -215,14 +215,14 @@ __global__ void __launch_bounds__(128 * kTcGroupsMax) k_push_sur(DevModel m, Pus
     }
     float in[3] = {0.0f, 0.0f, 0.0f}, out[3];
     if (live) {
-      step_sur_a<kPointForm<PREC, KERR, false>>(m, p, sc, ls);
+      step_sur_a<kGeoForm<PREC, KERR, false>>(m, p, sc, ls);
       in[0] = sc.a.in[0];
       in[1] = sc.a.in[1];
       in[2] = sc.a.in[2];
     }
     tc_mlp_eval(T, in, out);
     if (live) {
-      live = step_sur_b<PREC, kPointForm<PREC, KERR, false>>(m, io, p, sc, out, ls);
+      live = step_sur_b<PREC, kGeoForm<PREC, KERR, false>>(m, io, p, sc, out, ls);
       if (live && !in_grid(m, p.X)) {
         save_ph(io.pool, slot, p);
         unsigned long long o = atomicAdd(io.cnt + io.out_counter, 1ull);
