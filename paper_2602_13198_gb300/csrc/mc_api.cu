@@ -96,14 +96,14 @@ DevModel make_model(const mc_ctx *c) {
   m.a = p.a;
   m.mass = p.mass;
   m.hslope = p.hslope;
-  m.r_h = (p.mass > 0.0) ? 1.0 + std::sqrt(1.0 - p.a * p.a) : 0.0;
+  const double r_h = (p.mass > 0.0) ? 1.0 + std::sqrt(1.0 - p.a * p.a) : 0.0;
   double L = p.L_unit;
   m.L3 = L * L * L;
-  m.rho_unit = p.M_unit / m.L3;
-  m.B_unit = kCL * std::sqrt(4.0 * kPI * m.rho_unit);
-  m.Ne_unit = m.rho_unit / (kMP + kME);
-  m.Ccoef = kHPL * L / (kME * kCL * kCL);
-  m.fCcoef = (float)m.Ccoef;
+  const double rho_unit = p.M_unit / m.L3;
+  m.B_unit = kCL * std::sqrt(4.0 * kPI * rho_unit);
+  m.Ne_unit = rho_unit / (kMP + kME);
+  const double Ccoef = kHPL * L / (kME * kCL * kCL);
+  m.fCcoef = (float)Ccoef;
   m.R_high = p.R_high;
   m.R_low = p.R_low;
   m.gam = p.gam;
@@ -117,7 +117,7 @@ DevModel make_model(const mc_ctx *c) {
   m.verlet_tol = p.verlet_tol;
   m.verlet_maxit = p.verlet_maxit;
   m.r_record = p.r_record;
-  m.r_capture = (p.mass > 0.0) ? m.r_h * (1.0 + p.dh) : -1.0;
+  m.r_capture = (p.mass > 0.0) ? r_h * (1.0 + p.dh) : -1.0;
   m.bias_mode = p.bias_mode;
   m.bias_p0 = p.bias_p0;
   m.bias_max = p.bias_max;
@@ -150,7 +150,6 @@ DevModel make_model(const mc_ctx *c) {
   m.dx3 = c->dx3;
   m.x1_hi = c->x1_0 + c->n1 * c->dx1;
   m.ithetae_max = 1.0 / p.thetae_max;
-  m.iB_unit = 1.0 / m.B_unit;
   m.idx1 = 1.0 / c->dx1;
   m.idx2 = 1.0 / c->dx2;
   m.idx3 = 1.0 / c->dx3;
@@ -166,7 +165,7 @@ DevModel make_model(const mc_ctx *c) {
   m.kap_w = p.kappa > 0.0 ? (p.kappa - 3.0) / p.kappa : 0.0;
   m.gam2 = 2.0 * (p.gam - 1.0);
   m.cthe = (kMP / kME) * (p.gam - 1.0);
-  m.hCcoef = 0.5 * m.Ccoef;
+  m.hCcoef = 0.5 * Ccoef;
   m.a2 = p.a * p.a;
   m.twoa = 2.0 * p.a;
   m.M2 = 2.0 * p.mass;
@@ -213,7 +212,6 @@ DevModel make_model(const mc_ctx *c) {
   m.nF = c->nF;
   m.lnK2 = c->lnK2;
   m.nK2 = c->nK2;
-  m.hot = c->hot;
   m.start = c->start;
   m.zpref = c->zpref;
   m.zlnuc = c->zlnuc;

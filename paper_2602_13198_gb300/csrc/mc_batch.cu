@@ -210,7 +210,7 @@ static cudaError_t batch_enqueue(mc_ctx **ctxs, int n, const double *n_s, const 
   BatchKernel kern = pick_kernel(prec, sur, minb);
   const int smem = batch_smem_bytes(sur, minb);
   cudaFuncSetAttribute((const void *)kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  // shared memory over L1: the descriptors take ~48 KB, a CTA with four network row groups ~163 KB more
+  // shared memory over L1: the descriptors take 54 KB, a CTA with four network row groups ~163 KB more
   cudaFuncSetAttribute((const void *)kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
   void *args[] = {&b};
   if (timed) cudaEventRecord(bs->e0, st);

@@ -155,9 +155,15 @@ __device__ void batch_phase(const DevModel *sm, const BatchIO &b, const PushIO &
 
 // Dynamic shared memory of a batch CTA: the model descriptors, then (surrogate) the network's tiles.
 // Variants of 6 or more resident CTAs per SM (the double-float form, latency-bound, gains from resident
-// warps) read the descriptors from global memory through L1 instead: ~48 KB per CTA of shared memory
-// would cap residency at 4.
+// warps) read the descriptors from global memory through L1 instead: 54 KB per CTA of shared memory caps
+// residency at 4.  The descriptor stays small enough for that: with 896 bytes instead of 856 the 4-CTA variants
+// held 3 CTAs and paid their register cap for nothing, and the network's CTA came within 60 bytes a descriptor
+// of its limit.
 constexpr int kModelsSmem = (int)((sizeof(DevModel) * kMaxBatch + 127) / 128 * 128);
+// shared memory of an SM, its share reserved per CTA, the most of one CTA; kStaticSmem bounds k_batch's static part
+constexpr int kSmSmem = 228 * 1024, kCtaReserved = 1024, kCtaSmem = 227 * 1024, kStaticSmem = 1024;
+static_assert(4 * (kModelsSmem + kStaticSmem + kCtaReserved) <= kSmSmem, "four CTAs of the 4-CTA variants share an SM");
+static_assert(kModelsSmem + tc_smem_bytes(kTcGroupsMax) + kStaticSmem <= kCtaSmem, "the network variant fits a CTA");
 __host__ __device__ constexpr bool global_desc(bool sur, int minb) { return !sur && minb >= 6; }
 inline int batch_smem_bytes(bool sur, int minb) {
   return (global_desc(sur, minb) ? 0 : kModelsSmem) + (sur ? tc_smem_bytes(kTcGroupsMax) : 0);

@@ -302,10 +302,10 @@ __device__ __forceinline__ bool upper_half(double x) { return __double_as_longlo
 // ---------------------------------------------------------------- model view passed to kernels
 struct DevModel {
   // metric and units
-  double a, mass, hslope, r_h;
-  double rho_unit, B_unit, Ne_unit, Ccoef, L3;   // Ccoef = h L / (m_e c^2), L3 = L_unit^3
+  double a, mass, hslope;
+  double B_unit, Ne_unit, L3;   // L3 = L_unit^3
   double R_high, R_low, gam, thetae_min, thetae_max;
-  double ithetae_max, iB_unit;   // 1 / thetae_max, 1 / B_unit
+  double ithetae_max;   // 1 / thetae_max
   // emission band / weights
   double lnu_min, dlnu, dlntot;
   int n_nu;
@@ -332,7 +332,6 @@ struct DevModel {
   int nF;
   const double *lnK2;
   int nK2;
-  const double *hot;      // ln(sigma_h / sigma_T) [kHotNT][kHotNE]
   // per-run generation data
   const int64_t *start;   // exclusive scan of zone counts
   const double *zpref;    // 4 pi A nu_c per zone (int dOmega j_nu = zpref F(nu/nu_c))
@@ -340,7 +339,7 @@ struct DevModel {
   df dmass, da, dx1_0, dx1_hi, dr_record, dr_capture;   // double-float splits for the mixed geodesic
   df dpi2hh, dhh_pi, dd2th;   // pi (1 - h), (1 - h) / (2 pi), -2 pi^2 (1 - h): the theta map in double-float
   double kap_w;                // (kappa - 3) / kappa
-  double gam2, cthe, hCcoef;   // 2 (gam - 1), (m_p / m_e) (gam - 1), Ccoef / 2
+  double gam2, cthe, hCcoef;   // 2 (gam - 1), (m_p / m_e) (gam - 1), C / 2 with C = h L / (m_e c^2)
   double a2, twoa, M2, pi2hh, hh_pi2, d2th2;   // a^2, 2 a, 2 M and the theta map's pi (1-h), (1-h) / pi, -4 pi^2 (1-h)
   const df *dtab;             // double-float function table (kDfTabN entries)
   float fidx1, fidx2, fidx3, fx2_0, fx3_0;   // FP32 grid constants for the double-float zone lookup
