@@ -1,0 +1,34 @@
+"""Errors of the transport's FP64 functions against extended precision (numpy's long double), over the arguments
+that the kernels pass: within the bounds that follow from their roundings, and no further off than the
+functions that they took the place of."""
+import numpy as np
+import pytest
+
+from helpers import requires_gpu
+
+pytestmark = [pytest.mark.gpu, requires_gpu]
+LD = np.longdouble
+EPS = 2.0 ** -52
+N = 300000
+
+
+def evaluate(which, x):
+    from paper_2602_13198_gb300 import build, mc
+    build.build()
+    return mc.selftest_math(which, x)[0].astype(LD)
+
+
+def decades(rng, lo, hi):
+    return 10.0 ** rng.uniform(lo, hi, N)
+
+
+def ulp(ref):
+    return np.spacing(np.abs(ref.astype(np.float64)))
+
+
+def test_rsqrt():
+    rng = np.random.default_rng(1)
+    x = np.concatenate([decades(rng, -280, 280), rng.uniform(1.0, 4.0, N)])
+    ref = 1 / np.sqrt(x.astype(LD))
+    # the final rounding; the third-order remainder is below 0.02 ulp
+    assert (np.abs(evaluate(18, x) - ref) <= 0.55 * ulp(ref)).all()
