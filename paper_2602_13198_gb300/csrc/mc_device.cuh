@@ -109,8 +109,11 @@ __device__ __forceinline__ double exp_t(const double *T, double x) {
   return __hiloint2double(__double2hiint(y) + ((n >> 5) << 20), __double2loint(y));
 }
 
-// e^x from 2^(j/256): |r| <= ln2/512, so the series stops at r^4 (truncation below 4e-17) and the call takes 9
-// FP64 operations instead of 11; the 2 KB of table stay in L1.
+// e^x from 2^(j/256): |r| <= ln2/512 = b, so the series stops at r^4 and the call takes 9 FP64 operations instead
+// of 11; the 2 KB of table stay in L1.  The r^5/120 left out is replaced by the multiple of r^3 nearest to it on the
+// interval (0.84 b^2 r^3 / 120, Chebyshev's economization): 5e-18 remains instead of 4e-17, and the result is
+// within 1.03 ulp like exp_t's (1.31 with the plain series).
+constexpr double kExpQ3 = 1.0 / 6.0 + 0.84 * (0.6931471805599453 / 512.0) * (0.6931471805599453 / 512.0) / 120.0;
 __device__ __forceinline__ double exp_q(const double *T, double x) {
   if (!((__double_as_longlong(x) & 0x7fffffffffffffffLL) < 0x4086200000000000LL)) return exp(x);   // |x| < 708
   const double sh = 6755399441055744.0;
@@ -119,7 +122,7 @@ __device__ __forceinline__ double exp_q(const double *T, double x) {
   const double nd = t - sh;
   double r = fma(nd, -0.00270760617331689, x);
   r = fma(nd, -7.453964567463233e-13, r);
-  double q = fma(r, 1.0 / 24.0, 1.0 / 6.0);
+  double q = fma(r, 1.0 / 24.0, kExpQ3);
   q = fma(q, r, 0.5);
   const double pm1 = fma(q, r * r, r);
   const double tj = __ldg(T + kFtExpQ + (n & 255));

@@ -32,3 +32,11 @@ def test_rsqrt():
     ref = 1 / np.sqrt(x.astype(LD))
     # the final rounding; the third-order remainder is below 0.02 ulp
     assert (np.abs(evaluate(18, x) - ref) <= 0.55 * ulp(ref)).all()
+
+
+def test_exp():
+    rng = np.random.default_rng(2)
+    x = np.concatenate([-decades(rng, -16, 2.8), rng.uniform(-300, 20, N), rng.uniform(-1, 1, N)])
+    ref = np.exp(x.astype(LD))
+    # half an ulp each for the table and the result, 0.03 for the remainder of the series and the reduced argument
+    assert (np.abs(evaluate(11, x) - ref) <= 1.05 * ulp(ref)).all()
