@@ -223,11 +223,13 @@ int mc_fma_peak(int device, int dtype, double *flops);
  * double-float arithmetic, as the mixed-precision geodesic evaluates r = e^x1 (ref: CUDA exp,
  * |x| < 80); 4, 5: sin(pi x), cos(pi x) in double-float (ref: CUDA sincospi).  Inputs 3-5 are split
  * to double-float first and results joined back to double.  6: e^x and 7: ln x by the table-driven
- * FP64 functions of the FP64 transport (ref: CUDA exp, log); 8, 9: their sin(pi x), cos(pi x) (ref:
- * CUDA sincospi); 10: their e^x - 1 (ref: CUDA expm1); 11 to 15: e^x, ln x, sin(pi x), cos(pi x) and
- * e^x - 1 with the larger tables of the FP64 push (ref: CUDA's); 16: x^(1/6) from FP32 seeds (ref:
- * cbrt(sqrt(x))); 17, 18: 1 / x and x^(-1/2) from the hardware's seeds (ref: 1.0 / x, CUDA rsqrt); 19: the
- * bremsstrahlung rate at Theta_e = x and n_e = 1 from the tables (ref: the same fits with CUDA's functions).  x, y, ref are n host doubles (caller-owned).  Errors: INVALID_ARG, NO_DEVICE, CUDA. */
+ * FP64 functions of the emission and the component metric (ref: CUDA exp, log; no kernel calls 7 any more);
+ * 8, 9: their sin(pi x), cos(pi x) (ref: CUDA sincospi); 10: their e^x - 1 (ref: CUDA expm1); 11 to 15: e^x, ln x
+ * (as a table coordinate), sin(pi x), cos(pi x) and e^x - 1 with the larger tables of the FP64 push (ref:
+ * CUDA's); 16: x^(1/6) from FP32 seeds (ref: cbrt(sqrt(x))); 17, 18: 1 / x and x^(-1/2) from the hardware's
+ * seeds (ref: 1.0 / x, CUDA rsqrt); 19: the bremsstrahlung rate at Theta_e = x and n_e = 1 from the tables (ref:
+ * the same fits with CUDA's functions); 20, 21: ln x to half an ulp, for sampled variates and for table
+ * coordinates (ref: CUDA log).  x, y, ref are n host doubles (caller-owned).  Errors: INVALID_ARG, NO_DEVICE, CUDA. */
 int mc_selftest_math(int which, const double *x, double *y, double *ref, int64_t n);
 
 /* Zone superphoton counts for (N_s, seed) -- the same numbers mc_run computes and

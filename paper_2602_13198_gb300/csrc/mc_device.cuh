@@ -84,7 +84,9 @@ __device__ __forceinline__ double dmax_nn(double a, double b) {
 // mc_selftest_math.
 constexpr int kFtExp = 0, kFtInvC = 32, kFtLogHi = 160, kFtLogLo = 288, kFtSin = 416, kFtCos = 480;
 // larger tables of the push and generation kernels' exp_q, log_q (pairs) and sincospi_q (pairs)
-constexpr int kFtExpQ = 544, kFtExpm1Q = 800, kFtLogQ = 1056, kFtSinQ = 3104, kFtN = 7200;
+constexpr int kFtExpQ = 544, kFtExpm1Q = 800, kFtLogQ = 1056, kFtSinQ = 3104;
+constexpr int kFtLogN = 7200, kFtLogNLo = 9250, kFtN = 10275;   // log_n: 1025 pairs, 1025 low parts
+constexpr int kLogFold = 424;   // log_n takes c/2 from this node on (c = 1.4140625)
 void ftab_host(double *t);
 
 // e^x = 2^m 2^(j/32) e^r with x = (32 m + j) ln2/32 + r, |r| <= ln2/64 (n = 32 m + j by the 1.5 * 2^52
@@ -203,8 +205,11 @@ __device__ __forceinline__ double log_t(const double *T, double x) {
 }
 
 // log x with c = 1 + (j + 1/2)/1024 from the top 10 mantissa bits: |r| < 1/2048, series to r^4 (truncation below
-// 6e-18), ln2 and log c as single doubles: 9 FP64 operations instead of 15, absolute error within ~1 ulp of the
-// largest term (the callers interpolate tables in it).
+// 6e-18), ln2 and log c as single doubles: 9 FP64 operations instead of log_t's 15, absolute error within ~1 ulp of
+// the largest term and none of the relative accuracy near x = 1, so for coordinates of tables only (log_n elsewhere).
+// What is interpolated at these coordinates is no further off than with log_t: against quadruple precision sigma_h
+// has an RMS error of 2.9 epsilon (3.7 before) and G/K2 one of 7.4 (13.5), over Theta_e in [0.1, 1000],
+// eps in [1e-14, 100] and nu/nu_s in [1e-6, 1e4].
 __device__ __forceinline__ double log_q(const double *T, double x) {
   const long long b = __double_as_longlong(x);
   if (!(b >= 0x0010000000000000LL && b < 0x7FF0000000000000LL)) return log(x);
@@ -219,6 +224,35 @@ __device__ __forceinline__ double log_q(const double *T, double x) {
   const double l1p = fma(q, r * r, r);
   const double ed = __hiloint2double(0x43300000, (int)(0x80000000u + (unsigned)e)) - 4503601774854144.0;   // (double)e
   return fma(ed, 0.693147180559945309, tc.y) + l1p;
+}
+
+// log x = e ln2 - log v + log(1 + r), x = 2^e m and r = m v - 1: v is 1/c to 12 bits for the c = 1 + j/1024 nearest to m
+// (so that r is all but exact, |r| < 6.1e-4), and from c = 1.414 on 2^(e+1) and 2 v, so that nothing cancels
+// near x = 1.  ln2 and log v stand in a high part whose sum is exact and a low one: half an ulp, like CUDA's log, at
+// 10 FP64 operations instead of 28.7 with the series to r^4, whose remainder (below 1e-17) only shows within 1 % of
+// x = 1 (table coordinates), and at 12 with REL, which takes it to r^6 (sampled variates: up to 1.02 ulp where a step
+// of the table meets x = 1, the mean error CUDA's).
+constexpr double kLogN3 = 1.0 / 3.0 + 0.86 / (5.0 * 2048.0 * 2048.0);   // r^5/5 economized as in exp_q
+template <bool REL = false>
+__device__ __forceinline__ double log_n(const double *T, double x) {
+  const long long b = __double_as_longlong(x);
+  if (!(b >= 0x0010000000000000LL && b < 0x7FF0000000000000LL)) return log(x);
+  const int hi = (int)(b >> 32);
+  const int j = ((hi & 0x000fffff) + 512) >> 10;   // 0 .. 1024
+  const int e = (hi >> 20) - (j >= kLogFold ? 1022 : 1023);
+  const double m = __hiloint2double((hi & 0x000fffff) | 0x3ff00000, (int)b);
+  const double2 tv = __ldg(reinterpret_cast<const double2 *>(T + kFtLogN) + j);   // v, high part of -log v (or -log 2v)
+  const double r = fma(m, tv.x, -1.0);
+  double q;
+  if (REL) {
+    q = fma(fma(r, -1.0 / 6.0, 1.0 / 5.0), r, -0.25);
+    q = fma(fma(q, r, 1.0 / 3.0), r, -0.5);
+  } else {
+    q = fma(fma(r, -0.25, kLogN3), r, -0.5);
+  }
+  const double ed = __hiloint2double(0x43300000, (int)(0x80000000u + (unsigned)e)) - 4503601774854144.0;   // (double)e
+  const double kLn2Hi = 0.69314718055920821, kLn2Lo = 7.3710025651677989e-13;   // ln2: 40 significant bits + rest
+  return fma(ed, kLn2Hi, tv.y) + (fma(q, r * r, r) + fma(ed, kLn2Lo, __ldg(T + kFtLogNLo + j)));
 }
 
 // sin(pi x), cos(pi x) from a table of pi j/1024 (|pi r| <= pi/2048: two-term series, truncation below 2e-20): 14
@@ -1982,7 +2016,7 @@ __device__ __forceinline__ void thermal_electron(const double *T, double th, dou
     bool got;
     if (hot) {
       const double u1 = rng_u(s, seed), u2 = rng_u(s, seed), u3 = rng_u(s, seed), u4 = rng_u(s, seed);
-      const double p = -th * log_q(T, u1 * u2 * u3), eta = p - th * log_q(T, u4);
+      const double p = -th * log_n<true>(T, u1 * u2 * u3), eta = p - th * log_n<true>(T, u4);
       const double q = fma(p, p, 1.0);
       got = eta * eta - p * p > 1.0;
       gam = sqrt(q);
@@ -1992,11 +2026,10 @@ __device__ __forceinline__ void thermal_electron(const double *T, double th, dou
       double prod = 1.0;
       for (int i = 0; i < k; ++i) prod *= rng_u(s, seed);
       const double ua = rng_u(s, seed), ub = rng_u(s, seed);
-      double sz, cz;
-      sincospi_q(T, 2.0 * ub, sz, cz);
-      const double z2 = -2.0 * log_q(T, ua) * (cz * cz);
-      const double t = th * (0.5 * z2 - log_q(T, prod));
-      const double acc = (1.0 + t) * sqrt(t + 2.0) * rcp_n(1.4142135623730951 * (1.0 + 1.25 * t + 0.25 * t * t));
+      const double cz = cospi(2.0 * ub);
+      const double z2 = -2.0 * log_n<true>(T, ua) * (cz * cz);
+      const double t = th * (0.5 * z2 - log_n<true>(T, prod));
+      const double acc = (1.0 + t) * sqrt(t + 2.0) / (1.4142135623730951 * (1.0 + 1.25 * t + 0.25 * t * t));
       got = rng_u(s, seed) < acc;
       gam = 1.0 + t;
     }
@@ -2006,7 +2039,7 @@ __device__ __forceinline__ void thermal_electron(const double *T, double th, dou
     }
     mj = 0;
     mue = 2.0 * rng_u(s, seed) - 1.0;
-    beta = sqrt(1.0 - rcp_n(gam * gam));
+    beta = sqrt(1.0 - 1.0 / (gam * gam));
     const double om = 1.0 - beta * mue;
     const double acc = om * sigma_kn_ratio(eps * gam * om) * 0.5;
     if (rng_u(s, seed) < acc) return;

@@ -681,6 +681,11 @@ __global__ void k_selftest_math(int which, const double *x, double *y, double *r
     ref[i] = rsqrt(v);
     return;
   }
+  if (which == 20 || which == 21) {
+    y[i] = which == 20 ? log_n<true>(F, v) : log_n(F, v);
+    ref[i] = log(v);
+    return;
+  }
   if (which == 19) {
     y[i] = brems_q_t(F, 1.0, v);
     ref[i] = brems_q(1.0, v);
@@ -722,8 +727,8 @@ __global__ void k_selftest_math(int which, const double *x, double *y, double *r
   ref[i] = (which == 0) ? rs : rc;
 }
 
-// Tables of the exp, log and sincospi functions, in extended precision: 2^(j/32), 2^(j/256) and 2^(j/256) - 1; 1/c_j, log c_j split into its
-// double and the remainder (c_j = 1 + j/128); sin and cos (pi j/32), exact at multiples of pi/2.
+// Tables of the exp, log and sincospi functions, in extended precision: 2^(j/32), 2^(j/256) and 2^(j/256) - 1; 1/c_j and
+// log c_j of each logarithm; sin and cos of pi j/32 and pi j/1024, exact at multiples of pi/2.
 static void ftab_fill(double *t) {
   const long double pi = 3.141592653589793238462643383279502884L;
   for (int j = 0; j < 32; ++j) t[kFtExp + j] = (double)exp2l((long double)j / 32.0L);
@@ -735,6 +740,13 @@ static void ftab_fill(double *t) {
     const long double c = 1.0L + ((long double)j + 0.5L) / 1024.0L;
     t[kFtLogQ + 2 * j] = (double)(1.0L / c);
     t[kFtLogQ + 2 * j + 1] = (double)logl(c);
+  }
+  for (int j = 0; j <= 1024; ++j) {   // v = 1/c to 12 bits; -log v, or -log 2v from kLogFold on, high part a multiple of 2^-42
+    const long double v = rintl(4096.0L / (1.0L + (long double)j / 1024.0L)) / 4096.0L;
+    const long double l = -logl(j < kLogFold ? v : 2.0L * v), h = ldexpl(rintl(ldexpl(l, 42)), -42);
+    t[kFtLogN + 2 * j] = (double)v;
+    t[kFtLogN + 2 * j + 1] = (double)h;
+    t[kFtLogNLo + j] = (double)(l - h);
   }
   // sin(pi j/1024) for one octant pair, then by symmetry: exact at multiples of pi/2
   long double q[513];

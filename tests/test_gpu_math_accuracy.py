@@ -40,3 +40,17 @@ def test_exp():
     ref = np.exp(x.astype(LD))
     # half an ulp each for the table and the result, 0.03 for the remainder of the series and the reduced argument
     assert (np.abs(evaluate(11, x) - ref) <= 1.05 * ulp(ref)).all()
+
+
+@pytest.mark.parametrize("which,ulps,absolute", [(20, 1.1, 0.0), (21, 0.52, 1e-17)])
+def test_log(which, ulps, absolute):
+    rng = np.random.default_rng(3)
+    near = decades(rng, -15, -1)
+    x = np.concatenate([decades(rng, -14, 3), rng.uniform(0, 1, N), rng.uniform(0.9, 1.1, N), 1 - near, 1 + near,
+                        decades(rng, -300, 300), 1 + (np.arange(2048) + 0.5) / 2048, [1.0, 2.0, 0.5]])
+    ref = np.log(x.astype(LD))
+    y = evaluate(which, x)
+    # half an ulp of the result; within 1 % of x = 1 the variates' form has another half of the series' leading term,
+    # and the coordinates' form the remainder of its shorter series
+    assert (np.abs(y - ref) <= ulps * ulp(ref) + absolute).all()
+    assert y[-3] == 0.0 and (y[x < 1.0] <= absolute).all()
