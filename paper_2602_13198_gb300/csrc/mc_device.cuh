@@ -230,8 +230,8 @@ __device__ __forceinline__ double log_q(const double *T, double x) {
 // (so that r is all but exact, |r| < 6.1e-4), and from c = 1.414 on 2^(e+1) and 2 v, so that nothing cancels
 // near x = 1.  ln2 and log v stand in a high part whose sum is exact and a low one: half an ulp, like CUDA's log, at
 // 10 FP64 operations instead of 28.7 with the series to r^4, whose remainder (below 1e-17) only shows within 1 % of
-// x = 1 (table coordinates), and at 12 with REL, which takes it to r^6 (sampled variates: up to 1.02 ulp where a step
-// of the table meets x = 1, the mean error CUDA's).
+// x = 1 (table coordinates of the kappa population, bremsstrahlung), and everywhere at 14 with REL, which takes it to
+// r^6 and sums without the rounding of r (sampled variates).
 constexpr double kLogN3 = 1.0 / 3.0 + 0.86 / (5.0 * 2048.0 * 2048.0);   // r^5/5 economized as in exp_q
 template <bool REL = false>
 __device__ __forceinline__ double log_n(const double *T, double x) {
@@ -252,7 +252,10 @@ __device__ __forceinline__ double log_n(const double *T, double x) {
   }
   const double ed = __hiloint2double(0x43300000, (int)(0x80000000u + (unsigned)e)) - 4503601774854144.0;   // (double)e
   const double kLn2Hi = 0.69314718055920821, kLn2Lo = 7.3710025651677989e-13;   // ln2: 40 significant bits + rest
-  return fma(ed, kLn2Hi, tv.y) + (fma(q, r * r, r) + fma(ed, kLn2Lo, __ldg(T + kFtLogNLo + j)));
+  const double h = fma(ed, kLn2Hi, tv.y), l = fma(ed, kLn2Lo, __ldg(T + kFtLogNLo + j));
+  if (!REL) return h + (fma(q, r * r, r) + l);
+  const double s = h + r;   // h = 0 or |h| > |r|: the rounding of the sum is known exactly
+  return s + ((r - (s - h)) + fma(q, r * r, l));
 }
 
 // sin(pi x), cos(pi x) from a table of pi j/1024 (|pi r| <= pi/2048: two-term series, truncation below 2e-20): 14
@@ -2039,7 +2042,7 @@ __device__ __forceinline__ void thermal_electron(const double *T, double th, dou
     }
     mj = 0;
     mue = 2.0 * rng_u(s, seed) - 1.0;
-    beta = sqrt(1.0 - 1.0 / (gam * gam));
+    beta = sqrt(1.0 - rcp_n(gam * gam));
     const double om = 1.0 - beta * mue;
     const double acc = om * sigma_kn_ratio(eps * gam * om) * 0.5;
     if (rng_u(s, seed) < acc) return;
