@@ -54,3 +54,19 @@ def test_log(which, ulps, absolute):
     # and the coordinates' form the remainder of its shorter series
     assert (np.abs(y - ref) <= ulps * ulp(ref) + absolute).all()
     assert y[-3] == 0.0 and (y[x < 1.0] <= absolute).all()
+
+
+def test_bremsstrahlung_rate():
+    rng = np.random.default_rng(4)
+    th = np.concatenate([decades(rng, -3, 3), [1.0, np.nextafter(1.0, 0.0)]])
+    t, pi = th.astype(LD), LD("3.14159265358979323846264338327950288")
+    c = LD(7.2973525693e-3) * LD(9.1093837015e-28) * LD(2.99792458e10) ** 3
+    ei, ee = LD(1.25) * LD(6.6524587321e-25) * c, LD(2.8179403262e-13) ** 2 * c
+    with np.errstate(all="ignore"):
+        cold = (4 * np.sqrt(2 * t / pi ** 3) * (1 + LD(1.781) * t ** LD(1.34)) * ei + 20 / (9 * np.sqrt(pi))
+                * (44 - 3 * pi ** 2) * t * np.sqrt(t) * (1 + LD(1.1) * t + t * t - LD(1.25) * t * t * np.sqrt(t)) * ee)
+        hot = (9 * t / (2 * pi) * (np.log(LD(1.123) * t + LD(0.48)) + LD(1.5)) * ei
+               + 24 * t * (np.log(LD(1.1232) * t) + LD(1.28)) * ee)
+    ref = np.where(th < 1.0, cold, hot)
+    # five roundings of half an ulp on the longest path of the larger term, half of one from its constant
+    assert np.abs(evaluate(19, th) / ref - 1).max() <= 3 * EPS
