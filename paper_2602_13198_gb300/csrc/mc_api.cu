@@ -581,11 +581,18 @@ static double tune_next_scale(double s, int64_t carried, int64_t children, doubl
   return std::min(1e12, s * f);
 }
 
-// A generation (or a list handed back) of at most this many superphotons per warp of a full launch goes through
-// both phases in one launch.  Measured at 0 (never), 1, 2, 4, 8, 16 (ms a pass): the 64 x 32 sphere at N_s = 2000
-// 20.1, 17.7, 16.8, 16.7, 16.9, 16.7; the FP64 scattering sphere 91.7, 90.2, 90.5, 85.1, 84.8, 85.2; a 3-D torus at
-// N_s = 44000 38.9, 38.7, 37.7, 38.0, 39.4, 40.0 (more lanes of one warp in different phases).
-static const int64_t kSmallLanes = 4;
+// A generation (or a list handed back) of at most `small_lanes` superphotons per warp, of four warps per SM, goes through
+// both phases in one launch.  Four warps per SM leave each scheduler's pipe to one warp, so that the longest histories run
+// at the pace of one alone; eight warps with half the lanes each slowed them down.  Measured, ms a pass: every
+// generation through the phase kernels | eight warps per SM, 4 lanes | four warps, 2 lanes | four warps, 8 lanes:
+//   FP64: sphere 64 x 32, N_s = 2e3 20.3 | 16.8 | 17.6 | 16.8; sphere 1024 x 128, 1e6 89.7 | 81.7 | 85.7 | 79.1;
+//         torus a = 0.9375, 1e4 51.4 | 54.9 | 51.3 | 48.0; torus a = -0.94, 1e4 53.0 | 56.2 | 53.1 | 49.3; 3-D torus 51.3 | 50.8 | 49.1 | 48.6
+//   split: 12.8 | 9.6 | 10.2 | 9.6; 59.9 | 53.1 | 56.4 | 52.6; 33.3 | 33.8 | 33.3 | 31.6; 35.4 | 35.4 | 35.3 | 32.0; 30.0 | 28.9 | 28.6 | 28.0
+//   mixed: 7.4 | 5.0 | 5.5 | 4.9; 33.1 | 28.9 | 30.4 | 28.8; 22.1 | 25.8 | 22.1 | 25.4; 22.7 | 27.5 | 22.9 | 27.1; 21.6 | 20.8 | 20.1 | 21.2
+// (16 lanes: as 8, but the mixed torus at N_s = 3e4 33.6 for 27.5).  The mixed form with a != 0 gains from 2 lanes only: its
+// double-float step is bound by issue and instruction fetch, which the phase kernels' full warps use better.
+constexpr int64_t kSmallWarpsPerSm = 4;
+static int64_t small_lanes(int prec, bool kerr) { return prec == MC_PREC_MIXED && kerr ? 2 : 8; }
 static int push_small(mc_ctx *c, const DevModel &m, PushIO &pio, int prec, const int32_t *list, int64_t n, int64_t warps,
                       int block, cudaStream_t st) {
   pio.list_in = list;
@@ -607,8 +614,8 @@ static int transport(mc_ctx *c, int64_t u0, int64_t u1, const int64_t *uid_list_
   const bool tuning = tune && c->p.bias_target > 0.0;
   const int block = c->p.block ? c->p.block : 128;
   const int prec = c->p.precision;
-  int occ[3];   // resident CTAs per SM of the in-grid, free-streaming and both-phase kernels
-  for (int ph = 0; ph < 3; ++ph) {
+  int occ[2];   // resident CTAs per SM of the in-grid and free-streaming kernels
+  for (int ph = 0; ph < 2; ++ph) {
     occ[ph] = std::max(1, push_max_blocks_per_sm(prec, ph, block, m.a != 0.0 ? 1 : 0));
     if (c->p.ctas_per_sm > 0) occ[ph] = std::min(occ[ph], (int)c->p.ctas_per_sm);
   }
@@ -669,8 +676,10 @@ static int transport(mc_ctx *c, int64_t u0, int64_t u1, const int64_t *uid_list_
       int grid_init = (int)std::min<int64_t>((int64_t)c->sms * 4, (n_items + block - 1) / block);
       TIMED_LAUNCH(0, launch_init(m, iio, prec, grid_init, block, st));
       int64_t n_grid = (int64_t)c->cnt_host[CNT_L0], n_free = (int64_t)c->cnt_host[CNT_L1];
-      const int64_t warps = (int64_t)c->sms * occ[2] * (block / 32);
-      const auto small = [&](int64_t n) { return !use_sur && n <= kSmallLanes * warps; };
+      int64_t warps = c->sms * kSmallWarpsPerSm;
+      if (c->p.ctas_per_sm > 0) warps = std::min(warps, (int64_t)c->sms * c->p.ctas_per_sm * (block / 32));
+      const int64_t max_small = use_sur ? 0 : small_lanes(prec, m.a != 0.0) * warps;
+      const auto small = [&](int64_t n) { return n <= max_small; };
       if (small(n_items)) {   // both phases in one launch, spread over the warps
         rc = push_small(c, m, pio, prec, nullptr, n_items, warps, block, st);
         if (rc) return rc;
