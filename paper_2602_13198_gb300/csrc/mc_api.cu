@@ -518,7 +518,7 @@ int generate_async(mc_ctx *c, double n_s, uint64_t seed, cudaStream_t st) {
   cudaError_t e = cudaMemsetAsync(c->bad, 0, sizeof(int), st);
   if (e != cudaSuccess) return (int)e;
   launch_zone_prep(m, c->zvol, c->zpref, c->zlnuc, c->bad, st);
-  launch_weights(m, c->zvol, c->zpref, c->zlnuc, c->partial, c->nchunks, n_s, c->p.w_min, c->lnw, c->winv, st);
+  launch_weights(m, c->zvol, c->zpref, c->zlnuc, c->partial, c->nchunks, n_s, c->p.w_min, c->lnw, c->winv, c->sms, st);
   launch_counts(m, c->zvol, c->zpref, c->zlnuc, c->zgmax, c->znbar, c->counts, st);
   launch_scan(c->counts, c->start, c->bsum, c->nz, c->total_dev, st);
   c->last_seed = seed;

@@ -82,7 +82,7 @@ void launch_tables(const DevModel &m, double *lnF, double *lnFc, double *lnK2, d
 // generation (mc_tables.cu)
 void launch_zone_prep(const DevModel &m, double *zvol, double *zpref, double *zlnuc, int *bad, cudaStream_t st);
 void launch_weights(const DevModel &m, const double *zvol, const double *zpref, const double *zlnuc, double *partial,
-                    int nchunks, double n_s, double w_min, double *lnw, double *winv, cudaStream_t st);
+                    int nchunks, double n_s, double w_min, double *lnw, double *winv, int sms, cudaStream_t st);
 void launch_counts(const DevModel &m, const double *zvol, const double *zpref, const double *zlnuc, double *zgmax,
                    double *znbar, int64_t *counts, cudaStream_t st);
 void launch_scan(const int64_t *counts, int64_t *start, int64_t *bsum, int64_t n, int64_t *total_dev, cudaStream_t st);

@@ -123,7 +123,7 @@ extern "C" int mc_zone_counts_noalloc(mc_ctx *c, double n_s, uint64_t seed, int6
   e = cudaMemsetAsync(bad, 0, sizeof(int), st);
   if (e == cudaSuccess) {
     launch_zone_prep(m, zvol, zpref, zlnuc, bad, st);
-    launch_weights(m, zvol, zpref, zlnuc, partial, nchunks, n_s, c->p.w_min, lnw, winv, st);
+    launch_weights(m, zvol, zpref, zlnuc, partial, nchunks, n_s, c->p.w_min, lnw, winv, c->sms, st);
     launch_counts(m, zvol, zpref, zlnuc, zgmax, znbar, counts, st);
     launch_scan(counts, start, bsum, c->nz, total, st);
     k_flag_total<<<1, 32, 0, st>>>(bad, total);

@@ -411,11 +411,11 @@ __global__ void k_weight_final(DevModel m, const double *partial, int nchunks, d
 }
 
 void launch_weights(const DevModel &m, const double *zvol, const double *zpref, const double *zlnuc, double *partial,
-                    int nchunks, double n_s, double w_min, double *lnw, double *winv, cudaStream_t st) {
+                    int nchunks, double n_s, double w_min, double *lnw, double *winv, int sms, cudaStream_t st) {
   const bool thermal = !(m.kappa > 0.0) && !m.brems;
-  // eight nodes per CTA once that still leaves four CTAs per SM (152 SMs); one below, where the chip is not full
+  // eight nodes per CTA once that still leaves four CTAs per SM; one below, where the chip is not full
   // (16 chunks: 161 us before, 59 us with one node per CTA)
-  if ((int64_t)nchunks * m.n_nu >= 8 * 600) {
+  if ((int64_t)nchunks * m.n_nu >= 8 * 4 * (int64_t)sms) {
     const dim3 grid(nchunks, (m.n_nu + 7) / 8);
     if (thermal) k_weight_partial<true, 8><<<grid, 256, 0, st>>>(m, zvol, zpref, zlnuc, partial, nchunks);
     else k_weight_partial<false, 8><<<grid, 256, 0, st>>>(m, zvol, zpref, zlnuc, partial, nchunks);
