@@ -58,9 +58,7 @@ SURVEY = ("batched parameter survey: 64 synthetic 2-D Fishbone-Moncrief tori dra
 # Algorithmic operation counts (add/mul/div/sqrt = 1, FMA = 2, each transcendental = 1), itemised
 # from the formulas each kernel form evaluates.  The spin form is the one the library launches: the
 # Schwarzschild form (a = 0) leaves out the terms that vanish at a = 0; 3-D grids blend 8 corners.
-# The metric and acceleration are counted by components, a fixed unit of work per step; the FP64 geodesic
-# reaches the same values from the Kerr-Schild form with about a quarter of the operations, so its rate in
-# this unit can pass what the pipe executes.
+# First by metric components: the double-float geodesic, and the split form at a = 0.
 OPS_STEPSIZE = 10          # 1 / (|k1|/d1 + |k2|/d2 + |k3|/d3) in one division
 OPS_POSITION = 28          # x_{n+1} = x_n + k dl + dl^2/2 a (4 components) and the predictor start
 OPS_METRIC = {"kerr": 135, "schw": 59}      # metric, inverse and x1/x2 derivatives at x_{n+1}
@@ -76,18 +74,37 @@ OPS_CHILD_LOAD = 1500      # Compton kinematics at child load (tetrad, electron,
 OPS_EMIT = 2000            # emission: frequency and direction rejection, tetrad, k^mu
 
 
-def ops_grid_step(spin, dim):
-    """FP64 in-grid step outside the predictor loop."""
+# The Kerr-Schild point form, which the FP64 form runs at every spin and the split form's geodesic at a != 0.
+# Its termination and sign tests run on the integer pipes, its convergence test mostly in FP32.
+PT_STEPSIZE = 8            # (eps x2n) / ((|k1| + |k3|) x2n + |k2|)
+PT_POSITION = 25           # x_{n+1} = x_n + (k + a dl/2) dl (4 components) and the predictor start
+PT_POINT = {"kerr": 36, "schw": 29}         # r, theta map, sin and cos of theta, f, Sigma and the shared factors
+PT_PLASMA = {"kerr": 78, "schw": 72}        # the six products of U, B and k, u^t, b^2, eps, Theta_e
+PT_COEFF = 62              # nu, |B|, cos theta_B, j_nu (fit), B_nu, alpha_nu, cubic K2 and bilinear sigma_h cells
+PT_DEPTH = 11              # trapezoid optical depths, weight update, biased scattering depth
+PT_COMPONENTS = 14         # split form: metric components of the point for the FP32 coefficients
+PT_ACCEL = {"kerr": 66, "schw": 42}         # the Euler-Lagrange right-hand side in f, l and L
+PT_VERLET = 16             # k_{n+1} = k_n + (a_n + a_{n+1}) dl/2 and the differences of the convergence test
+
+
+def ops_grid_step(spin, dim, point=False):
+    """FP64 in-grid step outside the predictor loop: by metric components, or in the point form."""
+    if point:
+        return (PT_STEPSIZE + PT_POSITION + PT_POINT[spin] + OPS_INTERP[dim] + PT_PLASMA[spin] + PT_COEFF + PT_DEPTH)
     return (OPS_STEPSIZE + OPS_POSITION + OPS_METRIC[spin] + OPS_INTERP[dim] + OPS_PLASMA[spin] + OPS_COEFF
             + OPS_DEPTH + OPS_TERM)
 
 
-def ops_geodesic_step(spin):
+def ops_geodesic_step(spin, point=False):
     """Geodesic part of a step (the whole free-streaming step; the FP64-level part of a mixed step)."""
+    if point:
+        return PT_STEPSIZE + PT_POSITION + PT_POINT[spin]
     return OPS_STEPSIZE + OPS_POSITION + OPS_METRIC[spin] + OPS_TERM
 
 
-def ops_pass(spin):
+def ops_pass(spin, point=False):
+    if point:
+        return PT_ACCEL[spin] + PT_VERLET
     return OPS_ACCEL[spin] + OPS_VERLET
 
 
@@ -230,22 +247,35 @@ def sum_stats(stats):
     return out
 
 
-def fp64_roofline(st, spin, dim, fp64_peak, kernel, traffic_per_ph=None, hbm_peak=None, fp32_peak=None):
-    """In-grid FP64 kernel against the measured FP64 FMA peak: achieved = the itemised count of the
-    form that ran, by metric components, x the step, pass and event counters / the in-grid phase's event-timed
-    duration: work done per second, not instructions executed."""
-    t_grid = st["grid_ms"] / 1e3
-    ops = (ops_grid_step(spin, dim) * st["n_steps_grid"] + ops_pass(spin) * st["n_iters_grid"]
-           + OPS_EVENT * st["n_events"])
+def push_seconds(st):
+    """Seconds of both push phases (a small generation's one launch counts as in-grid time)."""
+    return (st["grid_ms"] + st["free_ms"]) / 1e3
+
+
+def fp64_roofline(st, spin, dim, fp64_peak, kernel, traffic_per_ph=None, hbm_peak=None, fp32_peak=None, point=False):
+    """FP64 kernels against the measured FP64 FMA peak.  point: the push kernels as they run, both phases: achieved =
+    the itemised count of the point form x the step, pass and event counters / the phases' event-timed duration.
+    Otherwise the in-grid phase alone, counted by metric components."""
+    if point:
+        t_grid = push_seconds(st)
+        ops = (ops_grid_step(spin, dim, True) * st["n_steps_grid"]
+               + ops_geodesic_step(spin, True) * (st["n_steps"] - st["n_steps_grid"])
+               + ops_pass(spin, True) * st["n_iters"] + OPS_EVENT * st["n_events"])
+    else:
+        t_grid = st["grid_ms"] / 1e3
+        ops = (ops_grid_step(spin, dim) * st["n_steps_grid"] + ops_pass(spin) * st["n_iters_grid"]
+               + OPS_EVENT * st["n_events"])
     ach = ops / t_grid
     r = {"bound": "alu", "achieved": ach / 1e12, "peak": fp64_peak / 1e12, "unit": "TFLOP/s", "frac": ach / fp64_peak,
          "traffic": None, "kernel": kernel,
-         "count": {"basis": "component form of the metric; the kernel's Kerr-Schild form executes fewer",
-                   "spin_form": spin, "grid_dim": dim, "ops_per_in_grid_step": ops_grid_step(spin, dim),
-                   "ops_per_predictor_pass": ops_pass(spin), "ops_per_event": OPS_EVENT,
-                   "in_grid_steps": st["n_steps_grid"], "predictor_passes": st["n_iters_grid"], "events": st["n_events"]},
+         "count": {"basis": "Kerr-Schild point form, as run" if point else "metric components",
+                   "spin_form": spin, "grid_dim": dim, "ops_per_in_grid_step": ops_grid_step(spin, dim, point),
+                   "ops_per_free_step": ops_geodesic_step(spin, point),
+                   "ops_per_predictor_pass": ops_pass(spin, point), "ops_per_event": OPS_EVENT,
+                   "in_grid_steps": st["n_steps_grid"], "predictor_passes": st["n_iters" if point else "n_iters_grid"],
+                   "events": st["n_events"]},
          "peak_source": "measured: project FP64 FMA-chain microbenchmark on this GPU (mc_fma_peak)",
-         "phase_s": {"init": st["init_ms"] / 1e3, "in_grid": t_grid, "free": st["free_ms"] / 1e3}}
+         "phase_s": {"init": st["init_ms"] / 1e3, "in_grid": st["grid_ms"] / 1e3, "free": st["free_ms"] / 1e3}}
     if fp32_peak:
         r["fp32_peak_tflops"] = fp32_peak / 1e12
     if traffic_per_ph and hbm_peak:
@@ -254,37 +284,36 @@ def fp64_roofline(st, spin, dim, fp64_peak, kernel, traffic_per_ph=None, hbm_pea
         r["traffic"] = tb
         r["traffic_note"] = ("ncu DRAM read+write per superphoton (%.1f B) x primaries handed to the first in-grid "
                              "launch of each run" % traffic_per_ph)
-        r["hbm"] = {"achieved_gbs": tb / t_grid / 1e9, "peak_gbs": hbm_peak, "frac": tb / t_grid / 1e9 / hbm_peak}
+        gbs = tb / (st["grid_ms"] / 1e3) / 1e9
+        r["hbm"] = {"achieved_gbs": gbs, "peak_gbs": hbm_peak, "frac": gbs / hbm_peak}
     return r
 
 
-def split_roofline(st, spin, fp64_peak, kernel, phase="in_grid"):
-    """Split form (FP64 geodesic, FP32 coefficients and weights) against the measured FP64 peak: achieved =
-    the FP64 geodesic operations of the in-grid phase / its duration (phase "batch": of every step over
-    the whole batched transport launch); the FP32 coefficient work rides on the FP32 pipes beside it."""
-    if phase == "in_grid":
-        ops = ops_geodesic_step(spin) * st["n_steps_grid"] + ops_pass(spin) * st["n_iters_grid"]
-        ach = ops / (st["grid_ms"] / 1e3)
-    else:
-        ops = ops_geodesic_step(spin) * st["n_steps"] + ops_pass(spin) * st["n_iters"]
-        ach = ops / (st["transport_ms"] / 1e3)
+def split_roofline(st, spin, fp64_peak, kernel, phase="push"):
+    """Split form (FP64 geodesic, FP32 coefficients and weights) against the measured FP64 peak: achieved = the FP64
+    geodesic operations of every step (point form at a != 0, metric components at a = 0) / the duration of the push
+    phases (phase "batch": of the whole batched transport launch, point form for every model); the FP32
+    coefficient work rides on the FP32 pipes beside it."""
+    pt = phase == "batch" or spin == "kerr"
+    ops = (ops_geodesic_step(spin, pt) * st["n_steps"] + (PT_COMPONENTS if pt else 0) * st["n_steps_grid"]
+           + ops_pass(spin, pt) * st["n_iters"])
+    ach = ops / (st["transport_ms"] / 1e3 if phase == "batch" else push_seconds(st))
     return {"bound": "alu", "kernel": kernel, "achieved": ach / 1e12, "peak": fp64_peak / 1e12, "unit": "TFLOP/s",
             "frac": ach / fp64_peak, "traffic": None,
             "peak_source": "measured: project FP64 FMA-chain microbenchmark on this GPU (mc_fma_peak)",
-            "count": {"ops_per_in_grid_step_fp64": ops_geodesic_step(spin), "ops_per_predictor_pass": ops_pass(spin),
-                      "in_grid_steps": st["n_steps_grid"], "predictor_passes": st["n_iters_grid"]}}
+            "count": {"basis": "Kerr-Schild point form" if pt else "metric components",
+                      "ops_per_step_fp64": ops_geodesic_step(spin, pt), "ops_per_predictor_pass": ops_pass(spin, pt),
+                      "steps": st["n_steps"], "in_grid_steps": st["n_steps_grid"], "predictor_passes": st["n_iters"]}}
 
 
-def df_roofline(st, spin, fp32_peak, fp64_peak, kernel, phase="in_grid"):
-    """Double-float kernel against the measured FP32 peak.  achieved = FP64-equivalent geodesic
-    operations x DF_FLOPS_PER_OP (an estimate from the library's double-float arithmetic); the ncu-measured
-    FP32-pipe busy fraction sits beside it."""
-    if phase == "in_grid":
-        ops = ops_geodesic_step(spin) * st["n_steps_grid"] + ops_pass(spin) * st["n_iters_grid"]
-        sec = st["grid_ms"] / 1e3
-    else:   # whole batched transport
-        ops = (ops_geodesic_step(spin) * st["n_steps"] + ops_pass(spin) * st["n_iters"]
-               + OPS_EMIT * st["n_emit"] + OPS_CHILD_LOAD * st["n_child"])
+def df_roofline(st, spin, fp32_peak, fp64_peak, kernel, phase="push"):
+    """Double-float kernels against the measured FP32 peak.  achieved = FP64-equivalent geodesic
+    operations of every step x DF_FLOPS_PER_OP (an estimate from the library's double-float arithmetic); the
+    ncu-measured FP32-pipe busy fraction sits beside it."""
+    ops = ops_geodesic_step(spin) * st["n_steps"] + ops_pass(spin) * st["n_iters"]
+    sec = push_seconds(st)
+    if phase == "batch":   # whole batched transport
+        ops += OPS_EMIT * st["n_emit"] + OPS_CHILD_LOAD * st["n_child"]
         sec = st["transport_ms"] / 1e3
     eq = ops / max(sec, 1e-30)
     fp32 = DF_FLOPS_PER_OP * eq
@@ -353,8 +382,8 @@ def config_forms(name, p, g, jobs, spin, dim, dev, timer, flush, peaks, weights,
         del m
     st0, sums0, ms0 = ref
     e = form_entry(st0, ms0)
-    e["roofline"] = fp64_roofline(st0, spin, dim, fp64_peak, "k_push_fp64<in-grid, %s>" % spin,
-                                  TRAFFIC_B_PER_PH.get((name, "fp64")), hbm_peak)
+    e["roofline"] = fp64_roofline(st0, spin, dim, fp64_peak, "k_push_fp64, k_push_small <%s>, both phases" % spin,
+                                  TRAFFIC_B_PER_PH.get((name, "fp64")), hbm_peak, point=True)
     if oracle_sums is not None and 1 in sums0:
         e["spectrum_error_vs_oracle"] = error_block([(sums0[1], oracle_sums)])
     out["plain_fp64"] = e
@@ -377,11 +406,11 @@ def config_forms(name, p, g, jobs, spin, dim, dev, timer, flush, peaks, weights,
         if oracle_sums is not None and 1 in sums:
             e["spectrum_error_vs_oracle"] = error_block([(sums[1], oracle_sums)])
         if prec == "split":
-            e["roofline"] = split_roofline(st, spin, fp64_peak, "k_push_%s<in-grid, %s> (FP64 geodesic, FP32 rest)"
+            e["roofline"] = split_roofline(st, spin, fp64_peak, "k_push_%s<%s>, both phases (FP64 geodesic, FP32 rest)"
                                            % ("sur" if sur else "split", spin))
         else:
             e["roofline"] = df_roofline(st, spin, fp32_peak, fp64_peak,
-                                        "k_push_%s<in-grid, %s> (double-float geodesic)" % ("sur" if sur else "mixed", spin))
+                                        "k_push_%s<%s>, both phases (double-float geodesic)" % ("sur" if sur else "mixed", spin))
         if sur:
             tf = FLOP_SUR_EVAL * st["n_steps_grid"] / (st["grid_ms"] / 1e3) / 1e12
             e["surrogate"] = {"tensor_achieved_tflops": tf, "bf16_peak_tflops": bf16_peak,
@@ -616,15 +645,15 @@ def main():
 
     share = 100 * st_main["grid_ms"] / max(st_main["transport_ms"], 1e-30)
     if args.main_precision == "mixed":
-        roofline = df_roofline(st_main, "kerr", fp32_peak, fp64_peak, "k_push_mixed<in-grid, kerr>: %.0f%% of transport "
-                               "time" % share)
+        roofline = df_roofline(st_main, "kerr", fp32_peak, fp64_peak, "k_push_mixed<kerr>, both phases (in-grid: %.0f%% "
+                               "of transport time)" % share)
     elif args.main_precision == "split":
-        roofline = split_roofline(st_main, "kerr", fp64_peak, "k_push_split<in-grid, kerr>: %.0f%% of transport time"
-                                  % share)
+        roofline = split_roofline(st_main, "kerr", fp64_peak, "k_push_split<kerr>, both phases (in-grid: %.0f%% of "
+                                  "transport time)" % share)
     else:
-        roofline = fp64_roofline(st_main, "kerr", 3, fp64_peak, "k_push_fp64<in-grid, kerr> (FP64, trilinear FP32 "
-                                 "fields): dominant kernel, %.0f%% of transport time" % share,
-                                 TRAFFIC_B_PER_PH.get(("c4", "fp64")), hbm_peak, fp32_peak)
+        roofline = fp64_roofline(st_main, "kerr", 3, fp64_peak, "k_push_fp64<kerr>, both phases (FP64, trilinear "
+                                 "FP32 fields): the dominant in-grid phase is %.0f%% of transport time" % share,
+                                 TRAFFIC_B_PER_PH.get(("c4", "fp64")), hbm_peak, fp32_peak, point=True)
 
     cpu = None
     oracle_c1_spec = None
