@@ -479,6 +479,30 @@ def survey_forms(args, dev, timer, flush, peaks, weights):
     return out
 
 
+def compact(line):
+    """The line for a reader that keeps only some kilobytes of output: of each configuration's forms the rate, its
+    ratio to plain FP64, the spectrum error and the fraction of peak; times to the microsecond."""
+    def form(f):
+        e, r = f.get("spectrum_error"), f.get("roofline")
+        out = {"value": float("%.4g" % f["value"])}
+        if "speedup_vs_plain_fp64" in f:
+            out["x_fp64"] = round(f["speedup_vs_plain_fp64"], 3)
+        if e:
+            out["lum_err"], out["within_1pct"] = float("%.2g" % e["total_luminosity_rel_max"]), e["within_1pct"]
+        if r:
+            out["frac"] = round(r["frac"], 4)
+        return out
+
+    out = dict(line)
+    if out.get("forms"):
+        out["forms"] = {c: ({k: (form(f) if isinstance(f, dict) and "value" in f else f) for k, f in v.items()
+                             if k != "workload"} if c != "peaks" else v) for c, v in out["forms"].items()}
+    if out.get("detail"):
+        out["detail"] = {k: ([round(t, 3) for t in v] if isinstance(v, list) else v) for k, v in out["detail"].items()
+                         if k != "generate_ms"}
+    return out
+
+
 # ---------------------------------------------------------------------------------------------
 def grid_dims(args):
     n1, n2, n3 = (int(x) for x in args.grid.split("x"))
@@ -540,6 +564,7 @@ def main():
     ap.add_argument("--no-forms", action="store_true", help="skip the per-configuration forms")
     ap.add_argument("--no-survey", action="store_true", help="skip the batched-survey form")
     ap.add_argument("--survey-scale", type=float, default=1.0, help="N_s multiplier of the survey form")
+    ap.add_argument("--full", action="store_true", help="print every counter of the forms (a line of some 50 KB)")
     ap.add_argument("--forms-scale", type=float, default=1.0, help="N_s multiplier of the 2-D configuration forms")
     args = ap.parse_args()
 
@@ -785,7 +810,7 @@ def main():
                            "step_ms": step_ms, "wall_s": t_wall,
                            "generate_ms": [s["generate_ms"] for s in stats],
                            "scatterings_per_s": st_main["n_events"] / dev_s}}
-        print(json.dumps(line), flush=True)
+        print(json.dumps(line if args.full else compact(line)), flush=True)
     if dist:
         dist.barrier()
         dist.destroy_process_group()
