@@ -589,8 +589,10 @@ static double tune_next_scale(double s, int64_t carried, int64_t children, doubl
 //         torus a = 0.9375, 1e4 51.4 | 54.9 | 51.3 | 48.0; torus a = -0.94, 1e4 53.0 | 56.2 | 53.1 | 49.3; 3-D torus 51.3 | 50.8 | 49.1 | 48.6
 //   split: 12.8 | 9.6 | 10.2 | 9.6; 59.9 | 53.1 | 56.4 | 52.6; 33.3 | 33.8 | 33.3 | 31.6; 35.4 | 35.4 | 35.3 | 32.0; 30.0 | 28.9 | 28.6 | 28.0
 //   mixed: 7.4 | 5.0 | 5.5 | 4.9; 33.1 | 28.9 | 30.4 | 28.8; 22.1 | 25.8 | 22.1 | 25.4; 22.7 | 27.5 | 22.9 | 27.1; 21.6 | 20.8 | 20.1 | 21.2
-// (16 lanes: as 8, but the mixed torus at N_s = 3e4 33.6 for 27.5).  The mixed form with a != 0 gains from 2 lanes only: its
-// double-float step is bound by issue and instruction fetch, which the phase kernels' full warps use better.
+// (16 lanes: as 8, but the mixed torus at N_s = 3e4 33.6 for 27.5).  With no more than one superphoton for each of eight
+// warps per SM, these are a little ahead: 37.4 for 38.1 on the torus at N_s = 2e3 in FP64, 23.5 for 23.9 split, 15.0
+// for 15.5 mixed.  The mixed form with a != 0 gains up to there only: its double-float step is bound by issue and
+// instruction fetch, which the phase kernels' full warps use better.
 constexpr int64_t kSmallWarpsPerSm = 4;
 static int64_t small_lanes(int prec, bool kerr) { return prec == MC_PREC_MIXED && kerr ? 2 : 8; }
 static int push_small(mc_ctx *c, const DevModel &m, PushIO &pio, int prec, const int32_t *list, int64_t n, int64_t warps,
@@ -598,6 +600,7 @@ static int push_small(mc_ctx *c, const DevModel &m, PushIO &pio, int prec, const
   pio.list_in = list;
   pio.list_out = nullptr;
   pio.n_in = n;
+  if (n <= 2 * warps && c->p.ctas_per_sm != 1) warps *= 2;
   pio.lanes = (int)((n + warps - 1) / warps);
   const int64_t per_cta = (int64_t)pio.lanes * (block / 32);
   TIMED_LAUNCH(1, launch_push(m, pio, prec, 2, (int)((n + per_cta - 1) / per_cta), block, st));
