@@ -233,7 +233,7 @@ __device__ __forceinline__ double log_q(const double *T, double x) {
 // (table coordinates of the kappa population, bremsstrahlung).  REL (sampled variates) takes it to r^6 and v = 1 for the
 // two nodes on either side of 1 (|r| < 2.5e-3), so that r is small beside the result elsewhere: within 0.67 ulp for
 // every x, the mean error CUDA's, at 12 operations.  Births of a mixed 3-D snapshot shard: 18.5 ms with log_q, 19.2 with
-// this, 22 with CUDA's log.
+// this, about 22 with CUDA's log (the pass took 157 ms for 153).
 constexpr double kLogN3 = 1.0 / 3.0 + 0.86 / (5.0 * 2048.0 * 2048.0);   // r^5/5 economized as in exp_q
 template <bool REL = false>
 __device__ __forceinline__ double log_n(const double *T, double x) {
@@ -2011,7 +2011,10 @@ __device__ __forceinline__ void boost3(R E, const R p[3], R beta, const R v[3], 
 // acceptance of compton_fluid in one loop, same draws in the same order.  Nested, a warp ran the inner loop to
 // its slowest lane once per outer proposal, and the cold branch recomputed its mixture weights each time (about
 // 16000 FP64 issues per warp of children); in one loop it waits for the lane with the most proposals once.  With
-// the scattering tetrad's shorter form, loading 360000 children of the 3-D snapshot went from 9.8 to 4.4 ms.
+// the scattering tetrad's shorter form, loading 360000 children of the 3-D snapshot went from 9.8 to 4.4 ms with
+// log_q's logarithms; log_n's cost is in its comment.  A NaN energy would never pass either acceptance: it ends at
+// the first proposal (none has been seen: no run of some hundred spheres and tori in any form reached the
+// proposal limit or had a non-finite wavevector).
 __device__ __forceinline__ void thermal_electron(const double *T, double th, double eps, Rng &s, uint64_t seed, double &gam,
                                                  double &mue, double &beta, int &rejcap) {
   const bool hot = th >= 0.25;
